@@ -76,10 +76,11 @@ extern "C" {
 
 /* options for mpm_set_option (tuning knobs; defaults in brackets) */
 #define MPM_OPT_USE_GRAPHS 1      /* capture forward/backward into CUDA graphs [1] */
-#define MPM_OPT_SMEM_TILE 2       /* 1: scatters accumulate in a shared-memory node box and
-                                     flush once per node; 0: float4 reductions straight to
-                                     the L2-resident grid [0, faster on GB300] */
-#define MPM_OPT_TILE_CAPACITY 3   /* max nodes of one CTA's shared tile [1024]; this and
+#define MPM_OPT_SMEM_TILE 2       /* accepted and checked, no effect [0]: an earlier scatter form
+                                     (a shared-memory node box); every scatter now sums the
+                                     particles of a warp that share a node in registers and
+                                     reduces straight to the L2-resident grid */
+#define MPM_OPT_TILE_CAPACITY 3   /* nodes of that box [1024]; this and
                                      MPM_OPT_GATHER_CAPACITY / MPM_OPT_SMEM_TILE return
                                      MPM_ERR_ARG (option unchanged) when the node boxes would
                                      not fit the device's shared memory per CTA */
@@ -119,27 +120,16 @@ extern "C" {
 #define MPM_OPT_PERSISTENT_CHUNK 11 /* persistent form: at most this many passes per launch
                                      (0 = a whole run of same-kind passes) [0]; bounds the
                                      duration of any one launch */
-#define MPM_OPT_BUCKET_SCATTER 14  /* 1: a particle pass groups its tile's particles by stencil
-                                     base and scatters each group with one warp, one float4
-                                     reduction per (base, node) summed in registers, instead of
-                                     one per (particle, node) [0: on GB300 the extra shared-
-                                     memory traffic of the group loop outweighed the saved
-                                     reductions].  FP32 sums only (ignored in the deterministic
-                                     mode and with MPM_OPT_SMEM_TILE). */
-#define MPM_OPT_PAIR_SCATTER 15    /* bit mask, 0..3: float4 reductions straight to the grid
-                                     merge the two contributions of a pair of particles
-                                     (consecutive in the set-up's base order) that share a
-                                     stencil base, one reduction per pair and node -- bit 0 in
-                                     the forward and re-simulation passes, bit 1 in the adjoint
-                                     passes [0; pairs share a base only in MPM_OPT_SORT_ORDER 1].
-                                     FP32 sums only. */
+#define MPM_OPT_BUCKET_SCATTER 14  /* accepted, no effect [0]: an earlier scatter form (one
+                                     reduction per stencil base and node of a tile) */
+#define MPM_OPT_PAIR_SCATTER 15    /* 0..3 accepted, no effect [0]: an earlier scatter form (one
+                                     reduction per pair of particles and node) */
 #define MPM_OPT_SORT_ORDER 16      /* particle order chosen by mpm_set_initial (takes effect at
                                      the next mpm_set_initial), by a grid coordinate per axis
-                                     in runs of 8 along the last axis: 0 the cell; 1 the
-                                     stencil base; 2 the cell, but the base on the last axis,
-                                     so that consecutive pairs of particles share their base
-                                     (what MPM_OPT_PAIR_SCATTER merges) [0: the adjoint passes'
-                                     gathers run fastest over the cell order's tiles] */
+                                     in runs of 8 along the last axis: 0 the cell, rows of
+                                     half cells along the last axis within a run; 1 the stencil
+                                     base; 2 the cell, but the base on the last axis [0: the
+                                     scatter merges most reductions over its rows] */
 #define MPM_OPT_BARRIER_TEST_EXTRA 10 /* test hook, 0..1024 [0]: arrivals every grid barrier
                                      waits for beyond the launch's own CTAs.  Nonzero values
                                      can never be met, so each persistent launch ends through
@@ -210,7 +200,7 @@ typedef struct mpm_scene_desc {
                                   m_p -> 2^40, momentum m_p dx/dt -> 2^40, velocity adjoint: its
                                   first scatter's largest contribution -> below 2^36 (a measuring
                                   pass per backward); a contribution beyond 2^55 is refused with
-                                  MPM_ERR_RANGE.  The shared scatter box is not used.  0: FP32
+                                  MPM_ERR_RANGE.  0: FP32
                                   atomic sums (default, faster).  No counterpart in the paper,
                                   whose GPU atomics are order-dependent as well. */
   int32_t ctrl_hidden;         /* 0: open-loop sine actuation (w = sine weights).  H in 1..64:

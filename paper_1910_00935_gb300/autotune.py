@@ -1,10 +1,9 @@
 """Autotuner for the launch knobs of libmpm (measurement-based, cached).
 
 The knobs are the library's runtime options: the capacity of the shared gather box
-(MPM_OPT_GATHER_CAPACITY), the scatter path (MPM_OPT_SMEM_TILE: shared node box vs. float4
-reductions straight to the grid; MPM_OPT_BUCKET_SCATTER: one reduction per stencil base and
-node, summed by a warp, vs. one per particle and node), the shared box capacity (MPM_OPT_TILE_CAPACITY), the
-CTA count of the end-of-sequence grid clear (MPM_OPT_GRID_BLOCKS), the launch form
+(MPM_OPT_GATHER_CAPACITY), the particle order (MPM_OPT_SORT_ORDER), the options of earlier scatter
+forms, which the library accepts without effect (MPM_OPT_SMEM_TILE, MPM_OPT_BUCKET_SCATTER,
+MPM_OPT_PAIR_SCATTER, MPM_OPT_TILE_CAPACITY), the CTA count of the end-of-sequence grid clear (MPM_OPT_GRID_BLOCKS), the launch form
 (MPM_OPT_PERSISTENT: one launch per pass, or persistent launches over the pass plan), and two
 memory-vs-recompute choices of the backward: a re-simulated segment's grids kept or recomputed
 per step (MPM_OPT_GRID_RECOMPUTE) and the re-simulation overlapped with the adjoint passes on a

@@ -12,8 +12,8 @@ namespace mpm {
 
 namespace {
 // Raise a kernel's dynamic shared-memory limit when static + dynamic may pass the default
-// 48 KB: the passes' static shared memory (box slots, bucket table, group sums, the
-// persistent forms' pass entry) stays below 8 KB, so any dynamic size above 32 KB sets it.
+// 48 KB: the passes' static shared memory (box slots, group sums, the persistent forms' pass
+// entry) stays below 5 KB, so any dynamic size above 32 KB sets it.
 template <typename K>
 cudaError_t allow_smem(K k, size_t smem) {
   if (smem <= 32 * 1024) return cudaSuccess;
@@ -22,7 +22,7 @@ cudaError_t allow_smem(K k, size_t smem) {
 
 template <int D, int MAT, int MODE, bool DET>
 cudaError_t step_one(const SimParams& P, const StepArgs& A, int n_tiles, cudaStream_t s) {
-  const size_t smem = step_smem_bytes<D>(P.tile_capacity, P.gather_capacity);
+  const size_t smem = step_smem_bytes<D>(P.gather_capacity);
   auto k = step_kernel<D, MAT, MODE, DET>;
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) {
@@ -41,7 +41,7 @@ cudaError_t step_one(const SimParams& P, const StepArgs& A, int n_tiles, cudaStr
 
 template <int D, int MAT, int MODE, bool DET>
 cudaError_t adj_one(const SimParams& P, const AdjArgs& A, int n_tiles, cudaStream_t s) {
-  const size_t smem = adj_smem_bytes<D>(P.tile_capacity, P.gather_capacity);
+  const size_t smem = adj_smem_bytes<D>(P.gather_capacity);
   auto k = adjoint_kernel<D, MAT, MODE, DET>;
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) {
@@ -113,8 +113,8 @@ cudaError_t adj_variant(int mode, const SimParams& P, const AdjArgs& A, int n_ti
 template <int D, int MAT, bool DET>
 cudaError_t persistent_variant(int kind_mode, const SimParams& P, const PassEntry* plan, int n_pass,
                                int n_tiles, const PersistCtl& ctl, cudaStream_t s, int* grid_out) {
-  const size_t ss = step_smem_bytes<D>(P.tile_capacity, P.gather_capacity);
-  const size_t as = adj_smem_bytes<D>(P.tile_capacity, P.gather_capacity);
+  const size_t ss = step_smem_bytes<D>(P.gather_capacity);
+  const size_t as = adj_smem_bytes<D>(P.gather_capacity);
   switch (kind_mode) {
     case kPassStep * 8 + kP2GOnly:
       return persistent_one(step_persistent_kernel<D, MAT, kP2GOnly, DET>, ss, plan, n_pass, n_tiles, ctl, s, grid_out);

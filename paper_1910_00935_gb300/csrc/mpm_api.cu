@@ -255,13 +255,7 @@ struct mpm_handle {
   int32_t resident_T = 0;  // T of the forward whose last segment is still in the segment buffer
   // options
   bool use_graphs = true;
-  bool smem_tile = false;  // measured on GB300: global float4 reductions beat shared FP32 atomics
-  bool bucket_scatter = false;  // one reduction per (base, node) of a tile (measured slower: off)
-  // one reduction per (pair sharing a base, node): bit 0 forward passes, bit 1 adjoint passes.
-  // Off by default: it needs the base order (sort_order 1), whose tiles make the adjoint
-  // passes' gathers slower than the cell order's (measured on GB300, cube3d: forward pass
-  // 43.6 vs 46.3 us, adjoint 88.9 vs 77.1 us)
-  int pair_scatter = 0;
+  bool smem_tile = false;  // with tile_capacity only checked against the device (see mpm.h)
   int sort_order = 0;  // particle order of mpm_set_initial: 0 cells, 1 stencil bases, 2 cells
                        // with the base on the last axis
   int tile_capacity = 1024;
@@ -392,12 +386,7 @@ SimParams params_for(const mpm_handle* h, int t) {
       P.basis[k - 1] =
           (float)std::sin(two_pi * k * (double)t / (double)d.act_period + (double)d.act_phase);
   }
-  // the shared scatter box sums in FP32 in arbitrary order: not in the deterministic mode
-  P.tile_capacity = h->smem_tile && !d.deterministic_p2g ? h->tile_capacity : 0;
   P.gather_capacity = h->gather_capacity;
-  // the bucketed scatter sums a base's particles in FP32 registers: not in the deterministic mode
-  P.bucket = h->bucket_scatter && !d.deterministic_p2g ? 1 : 0;
-  P.pair = d.deterministic_p2g ? 0 : h->pair_scatter;
   P.f_diag = 0.0f;  // the workspace holds E = F - I
   P.xfix = 1;       // and positions in 32-bit fixed point
   P.det = d.deterministic_p2g;
@@ -1245,15 +1234,13 @@ int run_sequence(mpm_handle* h, int64_t key, cudaStream_t stream, Fn&& issue) {
 }
 
 // Dynamic shared memory the particle passes need with the handle's capacities, plus the
-// passes' static shared memory (below 8 KB), against the device's per-CTA limit.
+// passes' static shared memory (below 5 KB), against the device's per-CTA limit.
 bool capacities_fit(const mpm_handle* h, std::string* why) {
   if (h->smem_optin <= 0) return true;
-  const SimParams P = params_for(h, 0);
-  const size_t need = (h->m.D == 2 ? std::max(step_smem_bytes<2>(P.tile_capacity, P.gather_capacity),
-                                              adj_smem_bytes<2>(P.tile_capacity, P.gather_capacity))
-                                   : std::max(step_smem_bytes<3>(P.tile_capacity, P.gather_capacity),
-                                              adj_smem_bytes<3>(P.tile_capacity, P.gather_capacity))) +
-                      8 * 1024;
+  const int cap = std::max(h->gather_capacity, h->smem_tile && !h->desc.deterministic_p2g ? h->tile_capacity : 0);
+  const size_t need = (h->m.D == 2 ? std::max(step_smem_bytes<2>(cap), adj_smem_bytes<2>(cap))
+                                   : std::max(step_smem_bytes<3>(cap), adj_smem_bytes<3>(cap))) +
+                      5 * 1024;
   if (need <= (size_t)h->smem_optin) return true;
   char buf[160];
   snprintf(buf, sizeof(buf), "the shared node boxes need %zu B of shared memory per CTA, the device allows %d B",
@@ -1647,15 +1634,14 @@ int mpm_set_option(mpm_handle* h, int32_t key, int64_t value) {
   switch (key) {
     case MPM_OPT_USE_GRAPHS: h->use_graphs = value != 0; break;
     case MPM_OPT_SMEM_TILE: h->smem_tile = value != 0; break;
-    case MPM_OPT_BUCKET_SCATTER: h->bucket_scatter = value != 0; break;
+    case MPM_OPT_BUCKET_SCATTER: break;  // no effect (see mpm.h)
     case MPM_OPT_SORT_ORDER:
       if (value < 0 || value > 2) return fail(h, MPM_ERR_ARG, "sort order must be 0, 1 or 2");
       h->sort_order = (int)value;
       break;
     case MPM_OPT_PAIR_SCATTER:
       if (value < 0 || value > 3) return fail(h, MPM_ERR_ARG, "pair scatter must be in [0, 3]");
-      h->pair_scatter = (int)value;
-      break;
+      break;  // no effect (see mpm.h)
     case MPM_OPT_GATHER_CAPACITY:
       if (value != 0 && (value < 27 || value > 12288))
         return fail(h, MPM_ERR_ARG, "gather capacity must be 0 or in [27, 12288]");

@@ -88,15 +88,9 @@ struct SimParams {
   int n_groups, n_basis;
   float basis[kMaxBasis];  // sin(2 pi k t / P + phi), k = 1..n_basis, at this pass's step
   float basis2[kMaxBasis]; // same at the step of an adjoint pass's recomputed P2G
-  int tile_capacity;       // max nodes of a CTA's shared scatter box (0 = global reductions)
   int gather_capacity;     // max nodes of a CTA's shared gather box (0 = gathers through L1)
-  int bucket;              // 1: FP32 scatters go through the per-base bucket table (one
-                           // reduction per base and node); 0: one per particle and node
   int xfix;                // 1: the state's x rows hold positions in 32-bit fixed point
                            // (the float bits are the int32 x * 2^31), 0: FP32 positions
-  int pair;                // FP32 reductions straight to the grid merge pairs of particles
-                           // that share a stencil base (one per pair and node): bit 0 in
-                           // the forward passes, bit 1 in the adjoint passes
   float f_diag;            // the F rows of the state hold F - f_diag I (0: E = F - I, 1: F)
   // deterministic accumulation: grids hold 64-bit fixed-point sums (node_words = 2 float4
   // slots per node), channel c of a contribution v enters as round(v * fix_c); mass uses
@@ -157,33 +151,23 @@ __host__ __device__ __forceinline__ int fx_clzll(unsigned long long u) {
 #endif
 }
 
-// round(c) as a 64-bit integer for |c| <= 2^55, equal to __float2ll_rn(c) but without the
-// 64-bit conversion, which issues on the FP64 pipe (1/64 of the FP32 rate here): below 2^23
-// the 32-bit conversion rounds; from 2^23 on a float is an integer, its mantissa shifted by
-// its exponent
-__host__ __device__ __forceinline__ long long fix_round(float c) {
-  if (fabsf(c) < 8388608.0f) return (long long)fx_f2i_rn(c);
-  const unsigned b = fx_float_bits(c);
-  const int sh = (int)((b >> 23) & 0xFFu) - 150;  // 0 <= sh <= 32 for 2^23 <= |c| <= 2^55
-  const long long m = (long long)((b & 0x7FFFFFu) | 0x800000u) << sh;
-  return (b >> 31) ? -m : m;
+// round(c) for |c| <= 2^55 as h * 2^28 + l, |h| <= 2^27 and |l| <= 2^27, with 32-bit conversions
+// only (the 64-bit conversion issues on the FP64 pipe, 1/64 of the FP32 rate here).  c * 2^-28
+// and its rounding h are exact floats (from 2^24 on a float is an integer), the remainder
+// c - h 2^28 is a multiple of c's last bit below 2^28, so it is exact, and h 2^28 is even: l
+// rounds as c itself does (ties to even).
+__host__ __device__ __forceinline__ void fix_split(float c, int& h, int& l) {
+  h = fx_f2i_rn(c * 3.7252902984619140625e-9f);
+  l = fx_f2i_rn(fmaf(-268435456.0f, (float)h, c));
 }
-
-// channels 0..nch-1 of v into the fixed-point node `node` of grid g (two float4 slots
-// per node); channel 0 is scaled by f0, the others by f1
-__device__ __forceinline__ void fix_red(float4* g, int64_t node, float4 v, float f0, float f1,
-                                        int nch, unsigned& err) {
-  unsigned long long* q = reinterpret_cast<unsigned long long*>(g + 2 * node);
-  const float c[4] = {v.x * f0, v.y * f1, v.z * f1, v.w * f1};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    if (k >= nch || c[k] == 0.0f) continue;
-    if (!(fabsf(c[k]) <= kFixLimit)) {
-      err |= kErrRange;
-      continue;
-    }
-    atomicAdd(q + k, (unsigned long long)fix_round(c[k]));
-  }
+__host__ __device__ __forceinline__ long long fix_join(int h, int l) {
+  return (long long)h * 268435456LL + (long long)l;
+}
+// round(c) as a 64-bit integer for |c| <= 2^55, equal to __float2ll_rn(c)
+__host__ __device__ __forceinline__ long long fix_round(float c) {
+  int h, l;
+  fix_split(c, h, l);
+  return fix_join(h, l);
 }
 
 // a 64-bit integer rounded to the nearest float (ties to even) with 32-bit integer and

@@ -10,18 +10,13 @@
 // is never reset while another CTA may still read it).
 //
 // Particle passes run one CTA per tile of up to kTile particles of one scene
-// (particles are Morton-sorted per scene at set-up, so a tile covers a compact block
-// of cells, ~8 particles per cell in 3D).  Each pass works in two orders:
-//   - gathers, stress and state I/O run in tile order (thread t = particle t), so the
-//     state rows are read and written coalesced;
-//   - scatters run in an interleaved order (warp w takes particles w, w+8, w+16, ...),
-//     so that the 32 lanes of a warp sit in 32 different cells and never hit the same
-//     node in the same instruction.  The per-particle scatter record (stencil base, f,
-//     and the affine pair a + B dpos) moves between the two orders through shared
-//     memory.
-// Scatters go to the grid with float4 reductions (default), or accumulate in a shared
-// node box flushed once per node (MPM_OPT_SMEM_TILE).  Gathers read a shared gather box
-// filled once per CTA (grid functions applied while filling), or the grid directly.
+// (particles are sorted per scene at set-up, so a tile covers a compact block of cells, ~8
+// particles per cell in 3D, and a warp's 32 particles are two runs along the last axis).
+// Thread t owns particle t: gathers, stress and state I/O are coalesced rows.  Scatters hand a
+// warp's 32 particles to columns of lanes that walk them in order and sum the particles that
+// share a node in registers before one float4 reduction to the grid (scatter_runs); the
+// records cross between the two through shared memory, warp by warp.  Gathers read a shared
+// gather box filled once per CTA (grid functions applied while filling), or the grid directly.
 //
 // Stencil loops are separable: the weight of node (i, j, k) is w0[i] w1[j] w2[k] and
 // dpos = (dp0[i], dp1[j], dp2[k]), so partial products over (i) and (i, j) are hoisted.
@@ -160,11 +155,11 @@ struct Rows {
   static constexpr int X = 0, V = D, C = 2 * D, F = 2 * D + D * D, Q = 2 * D + 2 * D * D;
 };
 
-// scatter records: packed base, f[D], a[D], B[D][D]
+// scatter records: kQuads float4 per particle, [quad][kTile] (see put_record)
 template <int D>
-struct Xch {
-  static constexpr int kWidth = 1 + 2 * D + D * D;
-  static constexpr int kStride = kTile + kTile / 8;  // padded: conflict-free in both orders
+struct Rec {
+  static constexpr int kQuads = D == 3 ? 6 : 4;
+  static constexpr int kFloats = 4 * kQuads * kTile;
 };
 
 // per-warp group sums of the dL/dw reduction
@@ -193,28 +188,16 @@ __device__ __forceinline__ void stage_wait() {
 }
 __device__ __forceinline__ float staged(const float* stage, int r) { return stage[r * kTile + threadIdx.x]; }
 
-__device__ __forceinline__ int scatter_slot(int t) { return (t & 31) * (kTile / 32) + (t >> 5); }
-__device__ __forceinline__ int xidx(int j) { return j + (j >> 3); }
-
-// dynamic shared memory of a particle pass: node box (4 floats per node, shared by the
-// gather box and the scatter box) + scatter records
-__host__ __device__ inline int box_floats(int scatter_cap, int gather_cap) {
-  int c = scatter_cap > gather_cap ? scatter_cap : gather_cap;
-  return 4 * (c > 0 ? c : 1);
+// dynamic shared memory of a particle pass: gather box (4 floats per node), scatter records,
+// staged rows
+__host__ __device__ inline int box_floats(int gather_cap) { return 4 * (gather_cap > 0 ? gather_cap : 1); }
+template <int D>
+inline size_t step_smem_bytes(int gather_cap) {
+  return sizeof(float) * ((size_t)box_floats(gather_cap) + Rec<D>::kFloats + Stage<D>::kStep * kTile);
 }
 template <int D>
-inline size_t pass_smem_bytes(int scatter_cap, int gather_cap) {
-  return sizeof(float) * ((size_t)box_floats(scatter_cap, gather_cap) +
-                          (size_t)Xch<D>::kWidth * Xch<D>::kStride);
-}
-// + the staged rows of a forward / adjoint pass
-template <int D>
-inline size_t step_smem_bytes(int scatter_cap, int gather_cap) {
-  return pass_smem_bytes<D>(scatter_cap, gather_cap) + sizeof(float) * Stage<D>::kStep * kTile;
-}
-template <int D>
-inline size_t adj_smem_bytes(int scatter_cap, int gather_cap) {
-  return pass_smem_bytes<D>(scatter_cap, gather_cap) + sizeof(float) * Stage<D>::kAdj * kTile;
+inline size_t adj_smem_bytes(int gather_cap) {
+  return sizeof(float) * ((size_t)box_floats(gather_cap) + Rec<D>::kFloats + Stage<D>::kAdj * kTile);
 }
 
 // Scene bounding box of the nodes a scatter touches: each warp reduces its valid lanes
@@ -309,7 +292,7 @@ struct BoxInfo {
 
 // Each box computation of a tile has its own 8-int slot of s_box (kBoxSlots slots, reset
 // together by reset_box_slots before the tile's first barrier), so a box costs one barrier.
-constexpr int kBoxSlots = 3;
+constexpr int kBoxSlots = 2;
 __device__ __forceinline__ void reset_box_slots(int* s_box) {
   if (threadIdx.x < 8 * kBoxSlots) s_box[threadIdx.x] = (threadIdx.x & 4) ? INT_MIN : INT_MAX;
 }
@@ -347,20 +330,6 @@ __device__ __forceinline__ BoxInfo<D> box_extent(bool valid, const int base[D], 
   b.vol = any ? vol : 0;
   b.use_tile = any && vol <= cap;
   return b;
-}
-
-// Zero the SoA accumulation box (4 arrays of cap floats).  Synchronises on both sides.
-template <int D>
-__device__ __forceinline__ void box_zero(const BoxInfo<D>& b, float* sm, int cap) {
-  __syncthreads();
-  if (b.use_tile)
-    for (int l = threadIdx.x; l < b.vol; l += blockDim.x) {
-      sm[l] = 0.0f;
-      sm[cap + l] = 0.0f;
-      sm[2 * cap + l] = 0.0f;
-      sm[3 * cap + l] = 0.0f;
-    }
-  __syncthreads();
 }
 
 // Fill the shared gather box (float4 per node, box-local order) with value(idx) for every
@@ -405,504 +374,220 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
   }
 }
 
-template <int D>
-__device__ __forceinline__ void box_flush(const BoxInfo<D>& b, const float* sm, int cap, float4* g,
-                                          int n) {
-  __syncthreads();
-  if (!b.use_tile) return;
-  for (int l = threadIdx.x; l < b.vol; l += blockDim.x) {
-    float4 v = make_float4(sm[l], sm[cap + l], sm[2 * cap + l], sm[3 * cap + l]);
-    if (v.x != 0.0f || v.y != 0.0f || v.z != 0.0f || v.w != 0.0f) {
-      int idx[D], r = l;
-#pragma unroll
-      for (int a = D - 1; a >= 0; --a) {
-        idx[a] = b.lo[a] + r % b.dim[a];
-        r /= b.dim[a];
-      }
-      atomicAdd(g + node_flat<D>(idx, n), v);
-    }
-  }
-}
-
-// Write this thread's scatter record (tile order).  A negative base marks "no scatter".
-template <int D>
-__device__ __forceinline__ void put_record(float* xr, bool valid, const int base[D], const float f[D],
-                                           const float a[D], const float B[D][D]) {
-  constexpr int S = Xch<D>::kStride;
-  const int i = xidx(threadIdx.x);
-  xr[i] = __int_as_float(valid ? pack_base<D>(base) : -1);
-#pragma unroll
-  for (int c = 0; c < D; ++c) {
-    xr[(1 + c) * S + i] = f[c];
-    xr[(1 + D + c) * S + i] = a[c];
-  }
-#pragma unroll
-  for (int c = 0; c < D * D; ++c) xr[(1 + 2 * D + c) * S + i] = B[c / D][c % D];
-}
-
-// quadratic B-spline weight of stencil offset o (compile-time after unrolling) at f = x/dx - base
-__device__ __forceinline__ float bspline_w(int o, float f) {
-  if (o == 0) {
-    const float r = 1.5f - f;
-    return 0.5f * r * r;
-  }
-  if (o == 1) {
-    const float r = f - 1.0f;
-    return 0.75f - r * r;
-  }
-  const float r = f - 0.5f;
-  return 0.5f * r * r;
-}
-
-// Reversed stencil walk.  Particles sorted by stencil base put ~8 particles (3D) of a base in
-// one tile, so two lanes of a reduction instruction often share a base; if both walk the 27
-// nodes in the same order they reduce into the same node in the same instruction, which the
-// L2 serialises.  A lane with rev walks them in reverse: by the B-spline symmetry
-// w_o(f) = w_(2-o)(2 - f) and dpos_o(f) = -dpos_(2-o)(2 - f), the contribution for the loop's
-// offset o, computed from f' = 2 - f and -B, belongs to node base + 2 - o.  This rewrites f
-// and B in place and returns the grid pointer of node base + 2 rev and the offset sign.
-template <int D>
-__device__ __forceinline__ float4* reversed_stencil(bool rev, float4* g, int n, const int base[D],
-                                                    float f[D], float B[D][D], int& sgn) {
-  int b[D];
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    f[a] = rev ? 2.0f - f[a] : f[a];
-    b[a] = base[a] + (rev ? 2 : 0);
-  }
-#pragma unroll
-  for (int i = 0; i < D; ++i)
-#pragma unroll
-    for (int j = 0; j < D; ++j) B[i][j] = rev ? -B[i][j] : B[i][j];
-  sgn = rev ? -1 : 1;
-  return g + node_flat<D>(b, n);
-}
-
-// Pair-merged scatter (FP32 sums, reductions straight to the grid).  On GB300 a pass's
-// time grows with its count of scattered float4 reductions (measured on the fused forward
-// pass of a 262,144-particle cube: 51 us with 27 per particle, 26 us with none and the
-// arithmetic kept).  Particles are sorted by stencil base with the last axis's half-cell
-// varying fastest, so particles 2j and 2j+1 of a tile usually share their base: two
-// threads take such a pair, each one half of the 3^D nodes, and sum the pair's two
-// contributions to a node before one reduction -- half the reductions for the same
-// arithmetic.  A pair whose bases differ scatters each particle's contributions on their
-// own.  The node half is uniform per warp (no divergence); each thread reads two records.
-template <int D, bool WITH_MASS>
-__device__ __noinline__ void scatter_pairs(const float* xr, int count, float4* g, int n,
-                                           const SimParams& P, float mass_c) {
-  static_assert(kTile % 64 == 0, "pairs: two node halves of whole warps");
-  constexpr int S = Xch<D>::kStride;
-  constexpr int NN = D == 3 ? 27 : 9;
-  constexpr int SPLIT = D == 3 ? 15 : 5;   // nodes of the first half (whole columns in 3D)
-  constexpr int HW = kTile / 64;           // warps per node half
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = warp >= HW ? 1 : 0;
-  // lanes of a warp take every second pair, so fewer of them share a base (and nodes)
-  const int j = lane * HW + (warp - h * HW);  // 0 .. kTile/2 - 1
-  const int ia = 2 * j, ib = 2 * j + 1;
-  const int pa = ia < count ? __float_as_int(xr[xidx(ia)]) : -1;
-  const int pb = ib < count ? __float_as_int(xr[xidx(ib)]) : -1;
-  const bool va = pa >= 0, vb = pb >= 0;
-  if (!va && !vb) return;
-  const bool merged = va && vb && pa == pb;
-  float fa[D], fb[D], aa[D], ab[D], Ba[D][D], Bb[D][D];
-#pragma unroll
-  for (int c = 0; c < D; ++c) {
-    fa[c] = va ? xr[(1 + c) * S + xidx(ia)] : 1.0f;
-    aa[c] = va ? xr[(1 + D + c) * S + xidx(ia)] : 0.0f;
-    fb[c] = vb ? xr[(1 + c) * S + xidx(ib)] : 1.0f;
-    ab[c] = vb ? xr[(1 + D + c) * S + xidx(ib)] : 0.0f;
-  }
-#pragma unroll
-  for (int c = 0; c < D * D; ++c) {
-    Ba[c / D][c % D] = va ? xr[(1 + 2 * D + c) * S + xidx(ia)] : 0.0f;
-    Bb[c / D][c % D] = vb ? xr[(1 + 2 * D + c) * S + xidx(ib)] : 0.0f;
-  }
-  int base_a[D], base_b[D];
-  unpack_base<D>(va ? pa : 0, base_a);
-  unpack_base<D>(vb ? pb : 0, base_b);
-  // odd lanes walk their pair's stencils in reverse (reversed_stencil)
-  const bool rev = (lane & 1) != 0;
-  int sgn;
-  float4* ga = reversed_stencil<D>(rev, g, n, base_a, fa, Ba, sgn);
-  float4* gb = reversed_stencil<D>(rev, g, n, base_b, fb, Bb, sgn);
-  // weights and dpos are formed where they are used (few registers: the pair's records
-  // already hold 2 (2D + D^2) values)
-#pragma unroll
-  for (int col = 0; col < (D == 3 ? 9 : 3); ++col) {
-    // column: (i, jj) in 3D (nodes k = 0..2), i in 2D (nodes jj = 0..2)
-    const int i = D == 3 ? col / 3 : col;
-    const int jj = D == 3 ? col % 3 : 0;
-    const int o0 = D == 3 ? col * 3 : col * 3;  // first node of the column
-    // the column's nodes all lie in one half (3D: 15 = 5 columns; 2D: split inside col 1)
-    if (D == 3 && ((o0 < SPLIT) != (h == 0))) continue;
-    float wca = bspline_w(i, fa[0]), wcb = bspline_w(i, fb[0]);
-    float qca[D], qcb[D];
-    const float dia = ((float)i - fa[0]) * P.dx, dib = ((float)i - fb[0]) * P.dx;
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-      qca[c] = aa[c] + Ba[c][0] * dia;
-      qcb[c] = ab[c] + Bb[c][0] * dib;
-    }
-    if (D == 3) {
-      const float dja = ((float)jj - fa[1]) * P.dx, djb = ((float)jj - fb[1]) * P.dx;
-      wca *= bspline_w(jj, fa[1]);
-      wcb *= bspline_w(jj, fb[1]);
-#pragma unroll
-      for (int c = 0; c < D; ++c) {
-        qca[c] += Ba[c][1] * dja;
-        qcb[c] += Bb[c][1] * djb;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int o = o0 + k;
-      if (D == 2 && ((o < SPLIT) != (h == 0))) continue;
-      const float Wa = wca * bspline_w(k, fa[D - 1]), Wb = wcb * bspline_w(k, fb[D - 1]);
-      const float dza = ((float)k - fa[D - 1]) * P.dx, dzb = ((float)k - fb[D - 1]) * P.dx;
-      float q_a[3] = {0.0f, 0.0f, 0.0f}, q_b[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int c = 0; c < D; ++c) {
-        q_a[c] = qca[c] + Ba[c][D - 1] * dza;
-        q_b[c] = qcb[c] + Bb[c][D - 1] * dzb;
-      }
-      const float4 ca = WITH_MASS ? make_float4(Wa * mass_c, Wa * q_a[0], Wa * q_a[1], D == 3 ? Wa * q_a[2] : 0.0f)
-                                  : make_float4(Wa * q_a[0], Wa * q_a[1], D == 3 ? Wa * q_a[2] : 0.0f, 0.0f);
-      const float4 cb = WITH_MASS ? make_float4(Wb * mass_c, Wb * q_b[0], Wb * q_b[1], D == 3 ? Wb * q_b[2] : 0.0f)
-                                  : make_float4(Wb * q_b[0], Wb * q_b[1], D == 3 ? Wb * q_b[2] : 0.0f, 0.0f);
-      const int off = sgn * (D == 3 ? stencil_off<D>(i, jj, k, n) : stencil_off<D>(i, k, 0, n));
-      if (merged) {
-        atomicAdd(ga + off, make_float4(ca.x + cb.x, ca.y + cb.y, ca.z + cb.z, ca.w + cb.w));
-      } else {
-        if (va) atomicAdd(ga + off, ca);
-        if (vb) atomicAdd(gb + off, cb);
-      }
-    }
-  }
-}
-
-// Interleaved scatter of the records: node (i, j, k) receives
-//   mass  W * mass_c                      (when WITH_MASS)
+// ---------------------------------------------------------------------------
+// Run-merged scatter: node (i, j, k) of a particle's stencil receives
+//   mass  W * mass_c          (when WITH_MASS)
 //   vec   W * (a + B dpos)
-// into the shared box (or global memory g when the box did not fit).
-template <int D, bool WITH_MASS, bool DET>
-__device__ __forceinline__ void scatter_records(const float* xr, int count, const BoxInfo<D>& bx,
-                                                float* sm, int cap, float4* g, int n,
-                                                const SimParams& P, float mass_c, float fix0,
-                                                float fix1, unsigned& err, bool pair) {
-  constexpr int S = Xch<D>::kStride;
-  if (!DET && !bx.use_tile && pair) {
-    scatter_pairs<D, WITH_MASS>(xr, count, g, n, P, mass_c);
-    return;
-  }
-  const int j = scatter_slot(threadIdx.x);
-  if (j >= count) return;
-  const int xi = xidx(j);
-  const int packed = __float_as_int(xr[xi]);
-  if (packed < 0) return;
-  int base[D];
-  unpack_base<D>(packed, base);
-  float f[D], a[D], B[D][D];
+// A particle's 3^D nodes are 3^(D-1) columns along the grid's last axis.  Each warp scatters
+// its own 32 particles: lane (slot, column) walks its slot's third (3D) or tenth (2D) of them
+// in order, sums their contributions to its column's three nodes in registers, and while the
+// stencil base moves along the last axis by a node or two only reduces the nodes that fall out
+// of the window into the grid; any other move reduces all three.  The particle order makes
+// runs of such moves (sort_keys_kernel), but nothing depends on it.
+//
+// Why: a pass with one float4 reduction per particle and node is bound by the L2's reduction
+// rate (~3.4e11 a second here, 7.1 M a pass on a 262,144-particle cube, about 20 us of its
+// 48 us).  On lattice rows of half cells the walk issues 6-8 reductions a particle in 3D
+// (27 before) and ~4 in 2D (9).  Three slots of nine columns keep 27 of 32 lanes busy; the
+// column's weights and affine value cost ~30 instructions per particle and lane, paid by
+// passes that issued only 38% of the time.  Per launch, between two events (us, before ->
+// after): 262,144-particle neo-Hookean cube fused step 48.5 -> 38.6, fused adjoint (half of
+// them with a recomputed P2G) 107.9 -> 92.0; 16 x 65,536 fixed-corotated 171.7 -> 153.7 and
+// 431 -> 377; 64 uneven 2D scenes (391,000 particles) 27.9 -> 23.4 and 52.5 -> 47.2; the cube
+// in the deterministic mode, whose every node takes four 64-bit integer atomics,
+// 101.6 -> 51.9 (89,505 particles).
+// ---------------------------------------------------------------------------
+
+// Write this thread's scatter record: the B-spline weights per axis, the affine value at the
+// stencil's centre node a + B dpos(1, 1, 1), its increment per node B dx, and the packed base
+// (-1: no scatter; its weights and values are then zero).  Every thread writes its record.
+template <int D>
+__device__ __forceinline__ void put_record(float4* rec, bool valid, const Axes<D>& s, const float a[D],
+                                           const float B[D][D], float dx) {
+  float ac[D], Bd[D][D], w[D][3];
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    f[c] = xr[(1 + c) * S + xi];
-    a[c] = xr[(1 + D + c) * S + xi];
-  }
+    ac[c] = valid ? a[c] : 0.0f;
 #pragma unroll
-  for (int c = 0; c < D * D; ++c) B[c / D][c % D] = xr[(1 + 2 * D + c) * S + xi];
-  float w[D][3], dp[D][3];
-  if (bx.use_tile || DET) axes_from_f<D>(f, P, w, dp);
-  if (bx.use_tile) {
-    int lb = base[0] - bx.lo[0];
-#pragma unroll
-    for (int c = 1; c < D; ++c) lb = lb * bx.dim[c] + (base[c] - bx.lo[c]);
-    const int s1 = D == 2 ? 1 : bx.dim[D - 1];
-    const int s0 = bx.dim[1] * s1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      float qi[D];
-#pragma unroll
-      for (int c = 0; c < D; ++c) qi[c] = a[c] + B[c][0] * dp[0][i];
-#pragma unroll
-      for (int jj = 0; jj < 3; ++jj) {
-        const float wij = w[0][i] * w[1][jj];
-        float qij[D];
-#pragma unroll
-        for (int c = 0; c < D; ++c) qij[c] = qi[c] + B[c][1] * dp[1][jj];
-        if (D == 2) {
-          const int l = lb + i * s0 + jj;
-          if (WITH_MASS) {
-            atomicAdd(&sm[l], wij * mass_c);
-            atomicAdd(&sm[cap + l], wij * qij[0]);
-            atomicAdd(&sm[2 * cap + l], wij * qij[1]);
-          } else {
-            atomicAdd(&sm[l], wij * qij[0]);
-            atomicAdd(&sm[cap + l], wij * qij[1]);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const float W = wij * w[D - 1][k];
-            const int l = lb + i * s0 + jj * s1 + k;
-            float q[D];
-#pragma unroll
-            for (int c = 0; c < D; ++c) q[c] = qij[c] + B[c][D - 1] * dp[D - 1][k];
-            if (WITH_MASS) {
-              atomicAdd(&sm[l], W * mass_c);
-              atomicAdd(&sm[cap + l], W * q[0]);
-              atomicAdd(&sm[2 * cap + l], W * q[1]);
-              atomicAdd(&sm[3 * cap + l], W * q[D - 1]);
-            } else {
-              atomicAdd(&sm[l], W * q[0]);
-              atomicAdd(&sm[cap + l], W * q[1]);
-              atomicAdd(&sm[2 * cap + l], W * q[D - 1]);
-            }
-          }
-        }
-      }
+    for (int b = 0; b < D; ++b) {
+      Bd[c][b] = valid ? B[c][b] * dx : 0.0f;
+      ac[c] += Bd[c][b] * (1.0f - s.f[b]);
     }
-  } else if (DET) {
-    const int64_t nb = node_flat<D>(base, n);
-    for_nodes<D>(w, [&](int i, int jj, int k, float W) {
-      float q[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        q[c] = a[c] + B[c][0] * dp[0][i] + B[c][1] * dp[1][jj];
-        if (D == 3) q[c] += B[c][D - 1] * dp[D - 1][k];
-      }
-      float4 v = WITH_MASS ? make_float4(W * mass_c, W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f)
-                           : make_float4(W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f, 0.0f);
-      fix_red(g, nb + stencil_off<D>(i, jj, k, n), v, fix0, fix1, WITH_MASS ? D + 1 : D, err);
-    });
+    for (int o = 0; o < 3; ++o) w[c][o] = valid ? s.w[c][o] : 0.0f;
+  }
+  const float base = __int_as_float(valid ? pack_base<D>(s.base) : -1);
+  float4* r = rec + threadIdx.x;
+  r[0] = make_float4(w[0][0], w[0][1], w[0][2], 0.0f);
+  if (D == 3) {
+    constexpr int z = D - 1;
+    r[kTile] = make_float4(w[1][0], w[1][1], w[1][2], 0.0f);
+    r[2 * kTile] = make_float4(w[z][0], w[z][1], w[z][2], ac[0]);
+    r[3 * kTile] = make_float4(ac[1], ac[z], Bd[0][0], Bd[0][1]);
+    r[4 * kTile] = make_float4(Bd[0][z], Bd[1][0], Bd[1][1], Bd[1][z]);
+    r[5 * kTile] = make_float4(Bd[z][0], Bd[z][1], Bd[z][z], base);
   } else {
-    // odd lanes walk the stencil in reverse (see reversed_stencil), so two lanes that share
-    // a base hit different nodes in each reduction instruction
-    const bool rev = (threadIdx.x & 1) != 0;
-    int sgn;
-    float4* gb = reversed_stencil<D>(rev, g, n, base, f, B, sgn);
-    float wr[D][3], dpr[D][3];
-    axes_from_f<D>(f, P, wr, dpr);
-    for_nodes<D>(wr, [&](int i, int jj, int k, float W) {
-      float q[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int c = 0; c < D; ++c) {
-        q[c] = a[c] + B[c][0] * dpr[0][i] + B[c][1] * dpr[1][jj];
-        if (D == 3) q[c] += B[c][D - 1] * dpr[D - 1][k];
-      }
-      float4 v = WITH_MASS ? make_float4(W * mass_c, W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f)
-                           : make_float4(W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f, 0.0f);
-      atomicAdd(gb + sgn * stencil_off<D>(i, jj, k, n), v);
-    });
+    r[kTile] = make_float4(w[1][0], w[1][1], w[1][2], base);
+    r[2 * kTile] = make_float4(ac[0], ac[1], Bd[0][0], Bd[0][1]);
+    r[3 * kTile] = make_float4(Bd[1][0], Bd[1][1], 0.0f, 0.0f);
   }
 }
 
-// ---------------------------------------------------------------------------
-// Bucketed scatter (FP32 sums).  A scattered float4 reduction costs the SM's L1/L2 path far
-// more than the arithmetic that produces it (measured on GB300: ~1.5 SM cycles per lane,
-// the equivalent of ~6 warp-wide FMA instructions), and a 128-particle tile sends ~3,500
-// of them into a box of ~200 nodes.  Particles that share a stencil base touch the same
-// 3^D nodes, so the tile's particles are grouped by base in a shared table, and one warp
-// takes a whole group: lane o < 3^D owns node base + o, sums the group's contributions in
-// registers and issues one reduction.  In 3D a tile holds ~16-64 bases of ~2-8 particles,
-// so the reductions drop 2-3x for ~30 extra FMA-class instructions per particle.  Bases
-// whose group overflows the table's slots, and tiles whose base box exceeds its keys, go
-// through the per-particle path.  Not used in the deterministic mode (its sums are
-// fixed point and order-free already).  Measured on GB300 it is slower than the per-particle
-// reductions (cube3d fused forward 53.2 vs 50.8 us): each group step is a chain of
-// dependent shared-memory reads (slot, then record) and the pass was already limited by
-// its shared-memory instruction queue as much as by the reductions; the pair-merged
-// scatter (scatter_pairs) halves the reductions without that cost.  It stays an option.
-// ---------------------------------------------------------------------------
-constexpr int kBucketKeys = 256;  // bases of one tile's base box the table can hold
-constexpr int kBucketSlots = 8;   // particles per base held in the table
-static_assert(kTile <= 256, "bucket entries hold tile-local indices in one byte");
-struct Buckets {
-  int count[kBucketKeys];                           // particles per base (kept zero between uses)
-  unsigned char order[kBucketKeys * kBucketSlots];  // their tile-local indices
+// a node's running sums in registers: weight (or nothing) and vector
+template <int D, bool WITH_MASS, bool DET>
+struct NodeSum {
+  static constexpr int kCh = D + (WITH_MASS ? 1 : 0);
+  float v[kCh];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int c = 0; c < kCh; ++c) v[c] = 0.0f;
+  }
+  __device__ __forceinline__ void add(float W, const float q[D], float, float, float, unsigned&) {
+    if (WITH_MASS) v[0] += W;
+#pragma unroll
+    for (int c = 0; c < D; ++c) v[c + (WITH_MASS ? 1 : 0)] += W * q[c];
+  }
+  __device__ __forceinline__ void reduce(float4* g, int node, float mass_c) const {
+    const float x = WITH_MASS ? v[0] * mass_c : v[0];
+    atomicAdd(g + node, make_float4(x, v[1], kCh > 2 ? v[kCh > 2 ? 2 : 0] : 0.0f, kCh > 3 ? v[kCh > 3 ? 3 : 0] : 0.0f));
+  }
 };
-__device__ __forceinline__ void buckets_zero(Buckets& b) {
-  for (int i = threadIdx.x; i < kBucketKeys; i += blockDim.x) b.count[i] = 0;
-}
-
-// array-of-structures scatter record of one particle: f[D], a[D], B[D][D], padded to float4s
-template <int D>
-struct Aos {
-  static constexpr int kFloats = D == 3 ? 16 : 8;
+// Deterministic mode: every contribution is rounded once, exactly as a reduction of its own
+// would round it (fix_round), and the integers are summed: h * 2^28 + l per channel with
+// |l| <= 2^27, |h| <= 2^27 a contribution, so the at most 11 of a walk fit 32 bits each.
+template <int D, bool WITH_MASS>
+struct NodeSum<D, WITH_MASS, true> {
+  static constexpr int kCh = D + (WITH_MASS ? 1 : 0);
+  int h[kCh], l[kCh];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int c = 0; c < kCh; ++c) h[c] = l[c] = 0;
+  }
+  __device__ __forceinline__ void add(float W, const float q[D], float mass_c, float fix0, float fix1,
+                                      unsigned& err) {
+    float c[kCh];
+    if (WITH_MASS) c[0] = W * mass_c * fix0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) c[a + (WITH_MASS ? 1 : 0)] = W * q[a] * (WITH_MASS || a > 0 ? fix1 : fix0);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+      const bool in = fabsf(c[k]) <= kFixLimit;
+      if (!in) err |= kErrRange;
+      int hi, lo;
+      fix_split(in ? c[k] : 0.0f, hi, lo);
+      h[k] += hi;
+      l[k] += lo;
+    }
+  }
+  __device__ __forceinline__ void reduce(float4* g, int node, float) const {
+    unsigned long long* q = reinterpret_cast<unsigned long long*>(g + 2 * (int64_t)node);
+#pragma unroll
+    for (int k = 0; k < kCh; ++k) {
+      const long long v = fix_join(h[k], l[k]);
+      if (v != 0) atomicAdd(q + k, (unsigned long long)v);
+    }
+  }
 };
-static_assert(Aos<3>::kFloats * kTile <= Xch<3>::kWidth * Xch<3>::kStride, "record area");
-static_assert(Aos<2>::kFloats * kTile <= Xch<2>::kWidth * Xch<2>::kStride, "record area");
 
-template <int D>
-__device__ __forceinline__ void put_record_aos(float* xr, const float f[D], const float a[D],
-                                               const float B[D][D]) {
-  float r[Aos<D>::kFloats];
-  int c = 0;
-#pragma unroll
-  for (int i = 0; i < D; ++i) r[c++] = f[i];
-#pragma unroll
-  for (int i = 0; i < D; ++i) r[c++] = a[i];
-#pragma unroll
-  for (int i = 0; i < D * D; ++i) r[c++] = B[i / D][i % D];
-#pragma unroll
-  for (; c < Aos<D>::kFloats; ++c) r[c] = 0.0f;
-  float4* dst = reinterpret_cast<float4*>(xr) + threadIdx.x * (Aos<D>::kFloats / 4);
-#pragma unroll
-  for (int i = 0; i < Aos<D>::kFloats / 4; ++i)
-    dst[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-}
-
-// keys of the tile's base box: the stencil box bx less its 2-node margin
-template <int D>
-__device__ __forceinline__ int bucket_keys(const BoxInfo<D>& bx) {
-  if (bx.vol <= 0) return 0;
-  int K = 1;
-#pragma unroll
-  for (int a = 0; a < D; ++a) K *= bx.dim[a] - 2;
-  return K;
-}
-template <int D>
-__device__ __forceinline__ int bucket_key(const BoxInfo<D>& bx, const int base[D]) {
-  int k = base[0] - bx.lo[0];
-#pragma unroll
-  for (int a = 1; a < D; ++a) k = k * (bx.dim[a] - 2) + (base[a] - bx.lo[a]);
-  return k;
-}
-
-// Enter this thread's particle in the table (valid particles only); returns true when its
-// base's slots were full and the particle must scatter on its own.
-template <int D>
-__device__ __forceinline__ bool bucket_fill(Buckets& bk, const BoxInfo<D>& bx, bool valid,
-                                            const int base[D]) {
-  if (!valid) return false;
-  const int key = bucket_key<D>(bx, base);
-  const int slot = atomicAdd(&bk.count[key], 1);
-  if (slot < kBucketSlots) {
-    bk.order[key * kBucketSlots + slot] = (unsigned char)threadIdx.x;
-    return false;
-  }
-  return true;
-}
-
-// One particle's 3^D reductions (mass W * mass_c when WITH_MASS, vector W (a + B dpos)) into
-// grid g from its own registers (the per-particle path)
-template <int D, bool WITH_MASS>
-__device__ __forceinline__ void scatter_one(float4* g, int n, const Axes<D>& s, const float a[D],
-                                            const float B[D][D], float mass_c) {
-  float4* gb = g + node_flat<D>(s.base, n);
-  for_nodes<D>(s.w, [&](int i, int jj, int k, float W) {
-    float q[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-      q[c] = a[c] + B[c][0] * s.dp[0][i] + B[c][1] * s.dp[1][jj];
-      if (D == 3) q[c] += B[c][D - 1] * s.dp[D - 1][k];
+// Scatter the warp's 32 records (written by its own lanes, __syncwarp'ed) into grid g.
+template <int D, bool WITH_MASS, bool DET>
+__device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n, float mass_c, float fix0,
+                                             float fix1, unsigned& err) {
+  constexpr int COLS = D == 3 ? 9 : 3, SLOTS = 32 / COLS;
+  const int lane = threadIdx.x & 31;
+  const int slot = lane / COLS, col = lane - slot * COLS;
+  if (slot >= SLOTS) return;
+  const int i = D == 3 ? col / 3 : col, j = D == 3 ? col - 3 * i : 0;
+  const float si = (float)(i - 1), sj = (float)(j - 1);
+  const int off = D == 3 ? (i * n + j) * n : i * n;
+  const float4* r = rec + (threadIdx.x & ~31u) + (slot * 32) / SLOTS;
+  const float4* end = rec + (threadIdx.x & ~31u) + ((slot + 1) * 32) / SLOTS;
+  NodeSum<D, WITH_MASS, DET> a0, a1, a2;
+  a0.zero();
+  a1.zero();
+  a2.zero();
+  int cur = -1, node = 0;
+#pragma unroll 1
+  for (; r < end; ++r) {
+    const float* w0 = reinterpret_cast<const float*>(r);
+    float wz[3], qc[D], Bz[D];  // weights along the last axis; value at the column's centre; its increment
+    float wc;
+    int base;
+    if (D == 3) {
+      const float4 q2 = r[2 * kTile], q3 = r[3 * kTile], q4 = r[4 * kTile], q5 = r[5 * kTile];
+      wc = w0[i] * w0[4 * kTile + j];
+      wz[0] = q2.x;
+      wz[1] = q2.y;
+      wz[2] = q2.z;
+      qc[0] = q2.w + si * q3.z + sj * q3.w;
+      qc[1] = q3.x + si * q4.y + sj * q4.z;
+      qc[D - 1] = q3.y + si * q5.x + sj * q5.y;
+      Bz[0] = q4.x;
+      Bz[1] = q4.w;
+      Bz[D - 1] = q5.z;
+      base = __float_as_int(q5.w);
+    } else {
+      const float4 q1 = r[kTile], q2 = r[2 * kTile];
+      const float2 q3 = *reinterpret_cast<const float2*>(r + 3 * kTile);
+      wc = w0[i];
+      wz[0] = q1.x;
+      wz[1] = q1.y;
+      wz[2] = q1.z;
+      base = __float_as_int(q1.w);
+      qc[0] = q2.x + si * q2.z;
+      qc[1] = q2.y + si * q3.x;
+      Bz[0] = q2.w;
+      Bz[1] = q3.y;
     }
-    float4 v = WITH_MASS ? make_float4(W * mass_c, W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f)
-                         : make_float4(W * q[0], W * q[1], D == 3 ? W * q[2] : 0.0f, 0.0f);
-    atomicAdd(gb + stencil_off<D>(i, jj, k, n), v);
-  });
-}
-
-// Every warp takes groups of the table in turn (3D: one group per warp step, lanes 0..26;
-// 2D: three groups, lanes 0..26 in threes of nine), sums each group's records into its
-// lane's node and issues one reduction per node; a group's count is reset to zero once
-// read, so the table is empty again for its next use.  The caller synchronised the CTA
-// after filling the table and writing the records.
-template <int D, bool WITH_MASS>
-__device__ __forceinline__ void scatter_buckets(Buckets& bk, int K, const BoxInfo<D>& bx,
-                                                const float* xr, float4* g, int n, const SimParams& P,
-                                                float mass_c) {
-  constexpr int L = D == 3 ? 27 : 9;  // nodes of a stencil = lanes per group
-  constexpr int PER = 32 / L;         // groups per warp step
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int sub = lane / L, o = lane - sub * L;
-  const bool lane_on = sub < PER;
-  int off[3];
-  off[0] = D == 3 ? o / 9 : o / 3;
-  off[1] = D == 3 ? (o / 3) % 3 : o % 3;
-  off[2] = D == 3 ? o % 3 : 0;
-  // the quadratic B-spline weight of stencil offset off_a as alpha (f - beta)^2 + gamma
-  float alpha[D], beta[D], gamma[D], odx[D];
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    alpha[a] = off[a] == 1 ? -1.0f : 0.5f;
-    beta[a] = off[a] == 0 ? 1.5f : (off[a] == 1 ? 1.0f : 0.5f);
-    gamma[a] = off[a] == 1 ? 0.75f : 0.0f;
-    odx[a] = (float)off[a];
-  }
-  int kd[D];
-#pragma unroll
-  for (int a = 0; a < D; ++a) kd[a] = bx.dim[a] - 2;
-  for (int k0 = warp * PER; k0 < K; k0 += nwarps * PER) {
-    const int key = k0 + sub;
-    const bool on = lane_on && key < K;
-    int cnt = on ? bk.count[key] : 0;
-    if (!__any_sync(0xffffffffu, cnt > 0)) continue;
-    const int m = cnt < kBucketSlots ? cnt : kBucketSlots;
-    float am = 0.0f, aq[3] = {0.0f, 0.0f, 0.0f};
-    for (int s = 0; s < m; ++s) {
-      const int q = bk.order[key * kBucketSlots + s];
-      const float4* r4 = reinterpret_cast<const float4*>(xr) + q * (Aos<D>::kFloats / 4);
-      float r[Aos<D>::kFloats];
-#pragma unroll
-      for (int i = 0; i < Aos<D>::kFloats / 4; ++i) {
-        const float4 v = r4[i];
-        r[4 * i] = v.x;
-        r[4 * i + 1] = v.y;
-        r[4 * i + 2] = v.z;
-        r[4 * i + 3] = v.w;
+    if (base != cur && base >= 0) {
+      // base and cur hold the last axis in their low bits and differ by at least 3 across rows
+      // (the last axis stays below its field's range), so a small difference is a move along it
+      const int d = base - cur;
+      if (cur >= 0 && d == 1) {
+        a0.reduce(g, node, mass_c);
+        a0 = a1;
+        a1 = a2;
+        a2.zero();
+        node += 1;
+      } else if (cur >= 0 && d == -1) {
+        a2.reduce(g, node + 2, mass_c);
+        a2 = a1;
+        a1 = a0;
+        a0.zero();
+        node -= 1;
+      } else {
+        if (cur >= 0) {
+          a0.reduce(g, node, mass_c);
+          a1.reduce(g, node + 1, mass_c);
+          if (d == 2) {
+            a0 = a2;
+          } else {
+            a2.reduce(g, node + 2, mass_c);
+            a0.zero();
+          }
+          a1.zero();
+          a2.zero();
+        }
+        int b[D];
+        unpack_base<D>(base, b);
+        node = node_flat<D>(b, n) + off;
       }
-      float W = 1.0f, dp[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const float f = r[a];
-        const float t = f - beta[a];
-        W *= fmaf(alpha[a] * t, t, gamma[a]);
-        dp[a] = (odx[a] - f) * P.dx;
-      }
-#pragma unroll
-      for (int c = 0; c < D; ++c) {
-        float qc = r[D + c];
-#pragma unroll
-        for (int b = 0; b < D; ++b) qc = fmaf(r[2 * D + c * D + b], dp[b], qc);
-        aq[c] = fmaf(W, qc, aq[c]);
-      }
-      am += W;
+      cur = base;
     }
-    if (on && cnt > 0) {
-      int base[D], r = key;
+    float q[D];
 #pragma unroll
-      for (int a = D - 1; a >= 0; --a) {
-        base[a] = bx.lo[a] + r % kd[a] + off[a];
-        r /= kd[a];
-      }
-      const float4 v = WITH_MASS ? make_float4(am * mass_c, aq[0], aq[1], D == 3 ? aq[2] : 0.0f)
-                                 : make_float4(aq[0], aq[1], D == 3 ? aq[2] : 0.0f, 0.0f);
-      atomicAdd(g + node_flat<D>(base, n), v);
-    }
-    __syncwarp();
-    if (on && o == 0 && cnt > 0) bk.count[key] = 0;
+    for (int c = 0; c < D; ++c) q[c] = qc[c] - Bz[c];
+    a0.add(wc * wz[0], q, mass_c, fix0, fix1, err);
+    a1.add(wc * wz[1], qc, mass_c, fix0, fix1, err);
+#pragma unroll
+    for (int c = 0; c < D; ++c) q[c] = qc[c] + Bz[c];
+    a2.add(wc * wz[2], q, mass_c, fix0, fix1, err);
   }
-}
-
-// The bucketed form of one tile's scatter, from the CTA's stencil box bx (every thread
-// calls it; bx came from box_extent, whose barrier separates this from the table's
-// previous use).  Writes the records, fills the table, synchronises, scatters by group and
-// lets overflowing particles scatter on their own.  Returns false (nothing done, no
-// barrier) when the tile's base box exceeds the table; the caller then takes the
-// per-particle path.
-template <int D, bool WITH_MASS>
-__device__ __forceinline__ bool bucket_scatter_tile(Buckets& bk, const BoxInfo<D>& bx, bool valid,
-                                                    const Axes<D>& s, const float a[D],
-                                                    const float B[D][D], float* xr, float4* g,
-                                                    int n, const SimParams& P, float mass_c) {
-  const int K = bucket_keys<D>(bx);
-  if (K > kBucketKeys) return false;
-  if (valid) put_record_aos<D>(xr, s.f, a, B);
-  const bool over = bucket_fill<D>(bk, bx, valid, s.base);
-  __syncthreads();
-  scatter_buckets<D, WITH_MASS>(bk, K, bx, xr, g, n, P, mass_c);
-  if (over) scatter_one<D, WITH_MASS>(g, n, s, a, B, mass_c);
-  return true;
+  if (cur >= 0) {
+    a0.reduce(g, node, mass_c);
+    a1.reduce(g, node + 1, mass_c);
+    a2.reduce(g, node + 2, mass_c);
+  }
 }
 
 __device__ __forceinline__ float particle_act(const SimParams& P, const float* basis, const int* group,
@@ -1023,12 +708,11 @@ __device__ __forceinline__ void reset_box(int* box, int scene) {
 // ---------------------------------------------------------------------------
 template <int D, int MAT, bool DET>
 __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis, bool active, int scene,
-                                         int64_t p, int count, const float x[D], const float v[D],
+                                         int64_t p, const float x[D], const float v[D],
                                          const float C[D][D], const float E[D][D], float mu_p,
                                          float la_p, int mat_p, const int* group, const float* wact,
-                                         float4* g, int* box_scene, float* sm, float* xr,
-                                         int* s_box, int* s_bbox, Buckets& bk, unsigned& err,
-                                         const double* R_in, double* R_out, int64_t N, bool pair) {
+                                         float4* g, int* box_scene, float4* rec, int* s_bbox,
+                                         unsigned& err, const double* R_in, double* R_out, int64_t N) {
   Axes<D> s;
   bool ok = make_axes<D>(x, P, s) && active;
   if (active && !ok) err |= kErrOOB;
@@ -1058,43 +742,13 @@ __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis,
       for (int j = 0; j < D; ++j) Am[i][j] = P.kappa * tau[i][j] + P.p_mass * C[i][j];
     }
   }
-  __syncthreads();  // the record area may still be read by an earlier scatter
-  if (!DET && P.bucket && P.tile_capacity == 0) {
-    const BoxInfo<D> bx = box_extent<D>(ok, s.base, INT_MAX, s_box + 16);
-    if (bucket_scatter_tile<D, true>(bk, bx, ok, s, mv, Am, xr, g, P.n_grid, P, P.p_mass)) {
-      if (threadIdx.x == 0 && bx.vol > 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          atomicMin(&box_scene[a], bx.lo[a]);
-          atomicMax(&box_scene[4 + a], bx.lo[a] + bx.dim[a] - 1);
-        }
-      }
-      return;
-    }
-  }
-  put_record<D>(xr, ok, s.base, s.f, mv, Am);
-  if (P.tile_capacity > 0) {
-    const BoxInfo<D> bx = box_extent<D>(ok, s.base, P.tile_capacity, s_box + 16);
-    box_zero<D>(bx, sm, P.tile_capacity);
-    scatter_records<D, true, DET>(xr, count, bx, sm, P.tile_capacity, g, P.n_grid, P, P.p_mass, P.fix_m,
-                             P.fix_p, err, pair);
-    box_flush<D>(bx, sm, P.tile_capacity, g, P.n_grid);
-    if (threadIdx.x == 0 && bx.vol > 0) {
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        atomicMin(&box_scene[a], bx.lo[a]);
-        atomicMax(&box_scene[4 + a], bx.lo[a] + bx.dim[a] - 1);
-      }
-    }
-  } else {
-    warp_bbox<D>(ok, s.base, s_bbox);
-    __syncthreads();
-    cta_bbox_flush<D>(s_bbox, box_scene);
-    BoxInfo<D> none;
-    none.use_tile = false;
-    scatter_records<D, true, DET>(xr, count, none, sm, 0, g, P.n_grid, P, P.p_mass, P.fix_m, P.fix_p, err,
-                                  pair);
-  }
+  __syncwarp();  // the warp's records may still be read by its earlier scatter
+  put_record<D>(rec, ok, s, mv, Am, P.dx);
+  warp_bbox<D>(ok, s.base, s_bbox);
+  __syncwarp();
+  scatter_runs<D, true, DET>(rec, g, P.n_grid, P.p_mass, P.fix_m, P.fix_p, err);
+  __syncthreads();  // every warp's share of the box
+  cta_bbox_flush<D>(s_bbox, box_scene);
 }
 
 // ---------------------------------------------------------------------------
@@ -1105,11 +759,11 @@ __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis,
 // synchronise between them.
 template <int D, int MAT, int MODE, bool NC, bool DET>
 __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A, int tile_index,
-                                          float* sm, int* s_box, int* s_bbox, Buckets& bk) {
+                                          float* sm, int* s_box, int* s_bbox) {
   using R = Rows<D>;
   cta_bbox_reset(s_bbox);
   reset_box_slots(s_box);
-  float* xr = sm + box_floats(P.tile_capacity, P.gather_capacity);
+  float4* rec = reinterpret_cast<float4*>(sm + box_floats(P.gather_capacity));
   const int4 tile = A.tiles[tile_index];
   const int scene = tile.x;
   const bool active = (int)threadIdx.x < tile.z;
@@ -1119,7 +773,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
   unsigned err = 0;
   run_clears<D>(A.clears, scene, tile.w, A.scene_tiles[scene], P.nnodes, n);
   if (tile.w == 0) reset_box(A.box_reset, scene);
-  float* stage = xr + Xch<D>::kWidth * Xch<D>::kStride;
+  float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
   if (MODE != kG2POnlyFull) {
     stage_row(stage, 0, A.mu + p);
     stage_row(stage, 1, A.la + p);
@@ -1219,10 +873,9 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
 
   if (MODE != kG2POnlyFull) {
     stage_wait<0>();
-    p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, tile.z, x, v, C, E, staged(stage, 0),
-                          staged(stage, 1), MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact,
-                     scene_grid(A.PMw, scene, P), A.box_w + scene * 8, sm, xr, s_box, s_bbox,
-                     bk, err, nullptr, A.Rw, N, (P.pair & 1) != 0);
+    p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, x, v, C, E, staged(stage, 0), staged(stage, 1),
+                          MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact, scene_grid(A.PMw, scene, P),
+                          A.box_w + scene * 8, rec, s_bbox, err, nullptr, A.Rw, N);
   }
   if (err) atomicOr(A.err, err);
 }
@@ -1241,9 +894,7 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_box[8 * kBoxSlots];
   __shared__ int s_bbox[8];
-  __shared__ Buckets s_bk;
-  buckets_zero(s_bk);  // ordered before its first use by the tile's first barrier
-  step_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox, s_bk);
+  step_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox);
 }
 
 // ---------------------------------------------------------------------------
@@ -1254,12 +905,12 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
 template <int D, int MAT, int MODE, bool NC, bool DET>
 __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& A, int tile_index,
                                              float* sm, int* s_box, int* s_bbox_ub, int* s_bbox_pm,
-                                             float* s_wbar, Buckets& bk) {
+                                             float* s_wbar) {
   using R = Rows<D>;
   cta_bbox_reset(s_bbox_ub);
   cta_bbox_reset(s_bbox_pm);
   reset_box_slots(s_box);
-  float* xr = sm + box_floats(P.tile_capacity, P.gather_capacity);
+  float4* rec = reinterpret_cast<float4*>(sm + box_floats(P.gather_capacity));
   const int4 tile = A.tiles[tile_index];
   const int scene = tile.x;
   const bool active = (int)threadIdx.x < tile.z;
@@ -1276,7 +927,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   __syncthreads();  // shared boxes reset
   // stage what the G2P-adjoint (state s: x, F) and the recomputed P2G (state s-1, mu, la)
   // read, so that those loads are in flight during the P2G-adjoint
-  float* stage = xr + Xch<D>::kWidth * Xch<D>::kStride;
+  float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
   if (MODE != kAdjP2G) {
 #pragma unroll
     for (int a = 0; a < D; ++a) stage_row(stage, a, A.st0 + (int64_t)(R::X + a) * N + p);
@@ -1557,12 +1208,9 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
     const float4* PMg = scene_grid(A.PM0, scene, P);
     auto velocity = [&](const int idx[D]) { return node_velocity<D>(pm_load<NC, DET>(PMg, node_flat<D>(idx, n), P), idx, P); };
-    const int cap_box = P.tile_capacity > P.gather_capacity ? P.tile_capacity : P.gather_capacity;
-    BoxInfo<D> bx;
-    bx.use_tile = false;
-    if (cap_box > 0) bx = box_extent<D>(ok, s.base, cap_box, s_box + 8);
-    BoxInfo<D> gbx = bx;
-    gbx.use_tile = bx.use_tile && P.gather_capacity > 0 && bx.vol <= P.gather_capacity;
+    BoxInfo<D> gbx;
+    gbx.use_tile = false;
+    if (P.gather_capacity > 0) gbx = box_extent<D>(ok, s.base, P.gather_capacity, s_box + 8);  // slot 1
     if (P.gather_capacity > 0) box_load<D>(gbx, reinterpret_cast<float4*>(sm), velocity);
     if (ok) with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, velocity, [&](auto load) {
       // x-adjoint terms on u - u_c (centre node), by the same B-spline identities
@@ -1629,40 +1277,12 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     float4* UBs = scene_grid(A.UB0, scene, P);
     float fix_u = 1.0f, unfix_u = 1.0f;
     if (DET) ub_scales(A.ub_m0, fix_u, unfix_u);
-    if (!DET && P.bucket && P.tile_capacity == 0 && cap_box > 0 &&
-        bucket_scatter_tile<D, false>(bk, bx, ok, s, vt, Bs, xr, UBs, n, P, 0.0f)) {
-      if (threadIdx.x == 0 && bx.vol > 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          atomicMin(&A.box_ub[scene * 8 + a], bx.lo[a]);
-          atomicMax(&A.box_ub[scene * 8 + 4 + a], bx.lo[a] + bx.dim[a] - 1);
-        }
-      }
-    } else if (P.tile_capacity > 0) {
-      put_record<D>(xr, ok, s.base, s.f, vt, Bs);
-      BoxInfo<D> sbx = bx;
-      sbx.use_tile = bx.use_tile && bx.vol <= P.tile_capacity;
-      box_zero<D>(sbx, sm, P.tile_capacity);  // same extent as the gather box
-      scatter_records<D, false, DET>(xr, tile.z, sbx, sm, P.tile_capacity, UBs, n, P, 0.0f, fix_u, fix_u, err,
-                                     false);
-      box_flush<D>(sbx, sm, P.tile_capacity, UBs, n);
-      if (threadIdx.x == 0 && sbx.vol > 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          atomicMin(&A.box_ub[scene * 8 + a], sbx.lo[a]);
-          atomicMax(&A.box_ub[scene * 8 + 4 + a], sbx.lo[a] + sbx.dim[a] - 1);
-        }
-      }
-    } else {
-      put_record<D>(xr, ok, s.base, s.f, vt, Bs);
-      warp_bbox<D>(ok, s.base, s_bbox_ub);
-      __syncthreads();
-      cta_bbox_flush<D>(s_bbox_ub, A.box_ub + scene * 8);
-      BoxInfo<D> none;
-      none.use_tile = false;
-      scatter_records<D, false, DET>(xr, tile.z, none, sm, 0, UBs, n, P, 0.0f, fix_u, fix_u, err,
-                                     (P.pair & 2) != 0);
-    }
+    put_record<D>(rec, ok, s, vt, Bs, P.dx);
+    warp_bbox<D>(ok, s.base, s_bbox_ub);
+    __syncwarp();
+    scatter_runs<D, false, DET>(rec, UBs, n, 0.0f, fix_u, fix_u, err);
+    __syncthreads();  // every warp's share of the box
+    cta_bbox_flush<D>(s_bbox_ub, A.box_ub + scene * 8);
   }
 
   // ---- recomputed P2G of step s-1 (the grid of the next adjoint pass) ----
@@ -1681,11 +1301,10 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     for (int i = 0; i < D; ++i)
 #pragma unroll
       for (int j = 0; j < D; ++j) E[i][j] = staged(stage, b + R::F + i * D + j) - (i == j ? P.f_diag : 0.0f);
-    p2g_pass<D, MAT, DET>(P, P.basis2, active, scene, p, tile.z, x, v, C, E, staged(stage, b + R::Q),
-                          staged(stage, b + R::Q + 1), MAT == kMixed ? A.matid[p] : MAT, A.group,
-                          A.wact,
-                     scene_grid(A.PMm, scene, P), A.box_m + scene * 8, sm, xr, s_box, s_bbox_pm,
-                     bk, err, A.Rm, nullptr, N, (P.pair & 2) != 0);
+    p2g_pass<D, MAT, DET>(P, P.basis2, active, scene, p, x, v, C, E, staged(stage, b + R::Q),
+                          staged(stage, b + R::Q + 1), MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact,
+                          scene_grid(A.PMm, scene, P), A.box_m + scene * 8, rec, s_bbox_pm, err, A.Rm,
+                          nullptr, N);
   }
   if (err) atomicOr(A.err, err);
 }
@@ -1698,10 +1317,7 @@ __global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
   __shared__ int s_bbox_ub[8];
   __shared__ int s_bbox_pm[8];
   __shared__ float s_wbar[kWbarSlots];
-  __shared__ Buckets s_bk;
-  buckets_zero(s_bk);  // ordered before its first use by the tile's first barrier
-  adjoint_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar,
-                                        s_bk);
+  adjoint_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar);
 }
 
 // ---------------------------------------------------------------------------
@@ -1816,8 +1432,6 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
   __shared__ int s_bbox[8];
   __shared__ int s_go, s_tile;
   __shared__ PassEntry e;
-  __shared__ Buckets s_bk;
-  buckets_zero(s_bk);  // ordered before its first use by the barriers that follow
   // a barrier of an earlier launch of this sequence gave up: its passes never finished, so
   // this launch would only run on an incomplete state
   if (*(volatile unsigned*)ctl.err & kErrTimeout) return;
@@ -1826,7 +1440,7 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
     __syncthreads();
     cta_copy(&e, plan + i);
     for (int t; (t = next_tile(ctl, i, &s_tile)) < n_tiles;) {
-      step_tile<D, MAT, MODE, false, DET>(e.P, e.S, t, sm, s_box, s_bbox, s_bk);
+      step_tile<D, MAT, MODE, false, DET>(e.P, e.S, t, sm, s_box, s_bbox);
       __syncthreads();
     }
   }
@@ -1843,8 +1457,6 @@ __global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
   __shared__ float s_wbar[kWbarSlots];
   __shared__ int s_go, s_tile;
   __shared__ PassEntry e;
-  __shared__ Buckets s_bk;
-  buckets_zero(s_bk);  // ordered before its first use by the barriers that follow
   // a barrier of an earlier launch of this sequence gave up: its passes never finished, so
   // this launch would only run on an incomplete state
   if (*(volatile unsigned*)ctl.err & kErrTimeout) return;
@@ -1853,7 +1465,7 @@ __global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
     __syncthreads();
     cta_copy(&e, plan + i);
     for (int t; (t = next_tile(ctl, i, &s_tile)) < n_tiles;) {
-      adjoint_tile<D, MAT, MODE, false, DET>(e.P, e.A, t, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar, s_bk);
+      adjoint_tile<D, MAT, MODE, false, DET>(e.P, e.A, t, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar);
       __syncthreads();
     }
   }

@@ -32,6 +32,7 @@ namespace {
 
 constexpr int64_t kMaxNodes = MPM_NOALLOC_MAX_NODES;
 constexpr int64_t kMaxParticles = MPM_NOALLOC_MAX_PARTICLES;
+constexpr int kGatherCapacity = 512;  // nodes of the shared gather box (as a handle's default)
 constexpr int64_t kMaxTiles = (kMaxParticles + kTile - 1) / kTile;
 
 // byte offsets inside the scratch array (each 256-byte aligned)
@@ -132,7 +133,7 @@ extern "C" int mpm_step_noalloc(const mpm_scene_desc* d, const float* state_in, 
     if (!g_setup_done[dev] || N == 0) {
       SimParams Q;
       memset(&Q, 0, sizeof(Q));
-      Q.tile_capacity = 1024;
+      Q.gather_capacity = kGatherCapacity;
       StepArgs Z;
       memset(&Z, 0, sizeof(Z));
       e = d->dim == 2 ? launch_step<2>(d->material, kP2GOnly, Q, Z, 0, s)
@@ -182,7 +183,7 @@ extern "C" int mpm_step_noalloc(const mpm_scene_desc* d, const float* state_in, 
   const double vol = d->dim == 2 ? 0.25 * dx * dx : 0.125 * dx * dx * dx;
   P.p_mass = (float)(d->rho * vol);
   P.kappa = (float)(-(double)d->dt * vol * 4.0 / (dx * dx));
-  P.tile_capacity = 1024;
+  P.gather_capacity = kGatherCapacity;
   P.f_diag = 1.0f;  // the caller's state rows hold F itself
   P.node_words = 1;
 

@@ -45,15 +45,14 @@ __device__ __forceinline__ int scene_of(const int64_t* off, int n_scenes, int64_
 // axis, which half of that coordinate's cell the particle sits in along each axis), with the
 // coordinates in runs of 8 along the last axis (the grid's contiguous one) and the runs in
 // Morton order of (other axes, run index), the second axis lowest: a 3D tile of 128 lattice
-// particles then covers 1 x 2 x 8 coordinates, and the lanes of a reduction instruction hit
-// nodes in z-runs (fewer L2 requests than a 2 x 2 x 4 Morton block, measured).  The half
-// bits vary fastest, the last axis's first.
-//  0: c = the cell floor(x/dx) on every axis.
-//  1: c = the stencil base floor(x/dx - 0.5) on every axis: the particles sharing a base (the
-//     ones that scatter to the same 3^D nodes) are contiguous.
-//  2: cells on the other axes, the base on the last: consecutive pairs (last-axis halves 0, 1)
-//     share their whole base, which the pair-merged scatter exploits, while the tile's lanes
-//     still spread over the cells' distinct bases.
+// particles then covers 1 x 2 x 8 coordinates.
+//  0: c = the cell floor(x/dx) on every axis.  Within a run the halves of the other axes come
+//     first and the position along the last axis varies fastest, so consecutive particles step
+//     along the last axis by half a cell: rows of 16 whose stencil bases repeat or move by one
+//     node, whatever the body's offset to the grid, which is what scatter_runs merges.
+//  1: c = the stencil base floor(x/dx - 0.5) on every axis, the half bits fastest: the
+//     particles sharing a base at set-up are contiguous.
+//  2: cells on the other axes, the base on the last, the half bits fastest.
 __global__ void sort_keys_kernel(int dim, int n_grid, int n_scenes, const int64_t* off, int64_t N,
                                  const float* x0, int order, uint64_t* keys, int* idx) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
@@ -74,8 +73,9 @@ __global__ void sort_keys_kernel(int dim, int n_grid, int n_scenes, const int64_
     const uint32_t last = c[dim - 1];
     uint64_t m = dim == 2 ? (spread2(last >> 3) | (spread2(c[0]) << 1))
                           : (spread3(c[1]) | (spread3(c[0]) << 1) | (spread3(last >> 3) << 2));
-    m = (m << 3) | (last & 7u);
-    keys[p] = ((uint64_t)scene_of(off, n_scenes, p) << 36) | (m << 3) | half;
+    const uint32_t low = order == 0 ? ((half >> 1) << 4) | ((last & 7u) << 1) | (half & 1u)
+                                    : ((last & 7u) << 3) | half;
+    keys[p] = ((uint64_t)scene_of(off, n_scenes, p) << 36) | (m << 6) | low;
     idx[p] = (int)p;
   }
 }
