@@ -20,8 +20,7 @@ namespace mpm {
 // Build-time launch shape (defaults measured on GB300): particles (= threads) per CTA of
 // the particle passes, and the CTAs per SM each pass is compiled to fit (register cap).
 // 128-particle tiles: measured 5-14% faster fwd+bwd than 256 (cube3d, robots3d, rects2d)
-// at the same register budget (80 per thread in the forward passes); the adjoint at 5 CTAs
-// per SM (96 registers) measured 1-6% faster than at 4 (128 registers).
+// at the same register budget (80 per thread in the forward passes).
 #ifndef MPM_TILE
 #define MPM_TILE 128
 #endif
@@ -44,8 +43,14 @@ namespace mpm {
 #ifndef MPM_POLAR_FP64
 #define MPM_POLAR_FP64 0
 #endif
-#ifndef MPM_ADJ_CTAS_PER_SM
-#define MPM_ADJ_CTAS_PER_SM (640 / MPM_TILE)  // 96 registers: a few spills, 25% more warps
+// adjoint passes: 2D 5 CTAs per SM (96 registers); 3D 4 (128 registers, no spills), which became
+// the faster one once the passes were shorter (fused adjoint, 262,144-particle neo-Hookean cube
+// 83 -> 81 us, 16 x 65,536 fixed-corotated 337 -> 318; in 2D 5 stays 10% faster)
+#ifndef MPM_ADJ_CTAS_PER_SM_2D
+#define MPM_ADJ_CTAS_PER_SM_2D (640 / MPM_TILE)
+#endif
+#ifndef MPM_ADJ_CTAS_PER_SM_3D
+#define MPM_ADJ_CTAS_PER_SM_3D (512 / MPM_TILE)
 #endif
 constexpr int kTile = MPM_TILE;   // particles (= threads) per CTA in particle passes
 static_assert(kTile % 32 == 0 && kTile >= 64 && kTile <= 1024, "tile must be whole warps");
@@ -306,20 +311,13 @@ __device__ __forceinline__ bool make_axes(const float* x, const SimParams& P, Ax
   return ok;
 }
 
-// weights only, from f (used by scatters that receive f from another thread)
-template <int D>
-__device__ __forceinline__ void axes_from_f(const float f[D], const SimParams& P, float w[D][3],
-                                            float dp[D][3]) {
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    float r0 = 1.5f - f[a], r1 = f[a] - 1.0f, r2 = f[a] - 0.5f;
-    w[a][0] = 0.5f * r0 * r0;
-    w[a][1] = 0.75f - r1 * r1;
-    w[a][2] = 0.5f * r2 * r2;
-    dp[a][0] = -f[a] * P.dx;
-    dp[a][1] = (1.0f - f[a]) * P.dx;
-    dp[a][2] = (2.0f - f[a]) * P.dx;
-  }
+// weight, its derivative and dpos of one axis at stencil offset o (a loop variable), with the
+// values make_axes forms
+__device__ __forceinline__ void axis_at(int o, float f, float dx, float& w, float& dw, float& dp) {
+  const float r = o == 1 ? f - 1.0f : (o == 0 ? 1.5f - f : f - 0.5f);
+  w = o == 1 ? 0.75f - r * r : 0.5f * r * r;
+  dw = o == 1 ? -2.0f * r : (o == 0 ? -r : r);
+  dp = ((float)o - f) * dx;
 }
 
 // ---------------------------------------------------------------------------

@@ -142,6 +142,9 @@ __device__ __forceinline__ float4 ub_load(const float4* g, int64_t node, const S
   }
   return grid_load<NC>(g + node);
 }
+struct NodePair {
+  float4 ub, pm;
+};
 // a scene's grid inside a buffer of per-scene grids
 __device__ __forceinline__ float4* scene_grid(float4* g, int scene, const SimParams& P) {
   return g + (int64_t)scene * P.nnodes * P.node_words;
@@ -200,34 +203,51 @@ inline size_t adj_smem_bytes(int gather_cap) {
   return sizeof(float) * ((size_t)box_floats(gather_cap) + Rec<D>::kFloats + Stage<D>::kAdj * kTile);
 }
 
-// Scene bounding box of the nodes a scatter touches: each warp reduces its valid lanes
-// into s_bbox (shared int atomics, native); after the CTA's next barrier thread 0 folds
-// s_bbox into the scene box with one set of global atomics (cta_bbox_flush).
-// s_bbox must have been reset (cta_bbox_reset) before a barrier preceding this call.
-__device__ __forceinline__ void cta_bbox_reset(int* s_bbox) {
-  if (threadIdx.x < 8) s_bbox[threadIdx.x] = (threadIdx.x & 4) ? INT_MIN : INT_MAX;
-}
+// Bounds of the stencil bases of a warp's valid lanes, written by lane 0 as two int4 (lo, hi) into
+// the warp's own slot, so that nothing has to be reset beforehand and no shared atomics are
+// needed; readers fold the warps' slots after the CTA's next barrier.
+constexpr int kWarps = kTile / 32;
+struct WarpBounds {
+  int4 lo[kWarps], hi[kWarps];
+};
+// static shared memory of a tile
+struct TileShared {
+  WarpBounds gather[2], scatter[2];  // at most two gathers and two scatters (adjoint passes)
+  int clear_box[8 * kMaxClears];     // scene boxes of the clear jobs
+};
 template <int D>
-__device__ __forceinline__ void warp_bbox(bool valid, const int base[D], int* s_bbox) {
-  const unsigned lane = threadIdx.x & 31u;
+__device__ __forceinline__ void warp_bounds(bool valid, const int base[D], WarpBounds& wb) {
+  int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    int lo = __reduce_min_sync(0xffffffffu, valid ? base[a] : INT_MAX);
-    int hi = __reduce_max_sync(0xffffffffu, valid ? base[a] + 2 : INT_MIN);
-    if (lane == 0 && hi >= lo) {
-      atomicMin(&s_bbox[a], lo);
-      atomicMax(&s_bbox[4 + a], hi);
-    }
+    lo[a] = __reduce_min_sync(0xffffffffu, valid ? base[a] : INT_MAX);
+    hi[a] = __reduce_max_sync(0xffffffffu, valid ? base[a] : INT_MIN);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    wb.lo[threadIdx.x >> 5] = make_int4(lo[0], lo[1], lo[2], 0);
+    wb.hi[threadIdx.x >> 5] = make_int4(hi[0], hi[1], hi[2], 0);
   }
 }
+
+// Thread a (lo) or 4 + a (hi), a < D, folds the CTA's bound (stencil bases wb, whose last node is
+// base + 2) into the scene box.  seen: that bound as the CTA read it when it started (box_seen);
+// one that it already covers needs no atomic.  (Six atomics of every CTA on one scene's box
+// serialise in the L2: they cost the plain P2G pass of a 2,048-tile cube 6 of 29 us.)
+__device__ __forceinline__ int box_seen(const int* bbox_scene) {
+  return threadIdx.x < 8 ? __ldcg(bbox_scene + threadIdx.x) : 0;
+}
 template <int D>
-__device__ __forceinline__ void cta_bbox_flush(const int* s_bbox, int* bbox_scene) {
-  if (threadIdx.x == 0 && s_bbox[4] >= s_bbox[0]) {
+__device__ __forceinline__ void cta_bbox_flush(const WarpBounds& wb, int* bbox_scene, int seen) {
+  if (threadIdx.x >= 8 || (threadIdx.x & 3) >= D) return;
+  const bool is_lo = threadIdx.x < 4;
+  const int* b = reinterpret_cast<const int*>(is_lo ? wb.lo : wb.hi) + (threadIdx.x & 3);
+  int v = b[0];
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      atomicMin(&bbox_scene[a], s_bbox[a]);
-      atomicMax(&bbox_scene[4 + a], s_bbox[4 + a]);
-    }
+  for (int w = 1; w < kWarps; ++w) v = is_lo ? min(v, b[4 * w]) : max(v, b[4 * w]);
+  if (is_lo) {
+    if (v != INT_MAX && v < seen) atomicMin(bbox_scene + threadIdx.x, v);
+  } else {
+    if (v != INT_MIN && v + 2 > seen) atomicMax(bbox_scene + threadIdx.x, v + 2);
   }
 }
 
@@ -262,22 +282,31 @@ __device__ __forceinline__ int stencil_off(int i, int j, int k, int n) {
   return D == 2 ? i * n + j : (i * n + j) * n + k;
 }
 
-// Calls fn(i, j, k, W) for the 3^D stencil nodes (k = 0 in 2D); indices are
-// compile-time after unrolling.
-template <int D, typename Fn>
-__device__ __forceinline__ void for_nodes(const float w[D][3], Fn&& fn) {
+// The gathers sum over a stencil axis by axis -- the last axis's three nodes, then the rows of a
+// plane, then the planes -- with the axis weights applied to the partial sums, so a node costs
+// its differences and the last axis's products only (3D: 9 multiply-adds a node for W d and its
+// moments against 15 with W formed per node).  In the 3D adjoint passes the planes run in a loop:
+// a third of the code and of the values in flight, which at 128 registers measured 5% faster on
+// 16 x 65,536 fixed-corotated particles (333 -> 316 us a fused pass) and 2% on the neo-Hookean
+// cube; unrolled, the forward passes' planes overlap and measured 1% faster.
+// wp: weight times dpos per axis (the first axis's come from axis_at).
+template <int D>
+struct GatherAxes {
+  float wp[D][3];
+  __device__ __forceinline__ explicit GatherAxes(const Axes<D>& s) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+    for (int a = 1; a < D; ++a)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const float wij = w[0][i] * w[1][j];
-      if (D == 2) {
-        fn(i, j, 0, wij);
-      } else {
+      for (int o = 0; o < 3; ++o) wp[a][o] = s.w[a][o] * s.dp[a][o];
+  }
+};
+
+template <int D>
+__device__ __forceinline__ bool is_wall(const int idx[D], const SimParams& P) {
+  bool wall = false;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) fn(i, j, k, wij * w[D - 1][k]);
-      }
-    }
+  for (int a = 0; a < D; ++a) wall = wall || (unsigned)(idx[a] - P.wall) >= (unsigned)(P.n_grid - 2 * P.wall);
+  return wall;
 }
 
 // ---------------------------------------------------------------------------
@@ -290,71 +319,82 @@ struct BoxInfo {
   bool use_tile;
 };
 
-// Each box computation of a tile has its own 8-int slot of s_box (kBoxSlots slots, reset
-// together by reset_box_slots before the tile's first barrier), so a box costs one barrier.
-constexpr int kBoxSlots = 2;
-__device__ __forceinline__ void reset_box_slots(int* s_box) {
-  if (threadIdx.x < 8 * kBoxSlots) s_box[threadIdx.x] = (threadIdx.x & 4) ? INT_MIN : INT_MAX;
-}
-
-// Extent of the node box covering the stencils of the CTA's valid particles.  Every
-// thread of the CTA must call this; s_box is a slot reset before an earlier barrier and
-// not used since.  Ends with a barrier, which also orders every earlier read of the
-// shared node box before the box_load that follows.
+// Extent of the node box covering the stencils of the CTA's valid particles.  Every thread of
+// the CTA must call this; wb has not been used since an earlier barrier.  Holds one barrier,
+// which also orders every earlier read of the shared node box before the box_load that follows.
 template <int D>
-__device__ __forceinline__ BoxInfo<D> box_extent(bool valid, const int base[D], int cap, int* s_box) {
-  const unsigned lane = threadIdx.x & 31u;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    int lo = valid ? base[a] : INT_MAX;
-    int hi = valid ? base[a] + 2 : INT_MIN;
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (lane == 0) {
-      atomicMin(&s_box[a], lo);
-      atomicMax(&s_box[4 + a], hi);
-    }
-  }
+__device__ __forceinline__ BoxInfo<D> box_extent(bool valid, const int base[D], int cap, WarpBounds& wb) {
+  warp_bounds<D>(valid, base, wb);
   __syncthreads();
+  int4 lo = wb.lo[0], hi = wb.hi[0];
+#pragma unroll
+  for (int w = 1; w < kWarps; ++w) {
+    const int4 l = wb.lo[w], h = wb.hi[w];
+    lo = make_int4(min(lo.x, l.x), min(lo.y, l.y), min(lo.z, l.z), 0);
+    hi = make_int4(max(hi.x, h.x), max(hi.y, h.y), max(hi.z, h.z), 0);
+  }
+  const int l3[3] = {lo.x, lo.y, lo.z}, h3[3] = {hi.x, hi.y, hi.z};
+  const bool any = hi.x >= lo.x;
   BoxInfo<D> b;
   int vol = 1;
-  bool any = true;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    b.lo[a] = s_box[a];
-    int hi = s_box[4 + a];
-    any = any && hi >= b.lo[a];
-    b.dim[a] = any ? hi - b.lo[a] + 1 : 0;
+    b.lo[a] = l3[a];
+    b.dim[a] = any ? h3[a] - l3[a] + 3 : 0;
     vol *= b.dim[a];
   }
-  b.vol = any ? vol : 0;
+  b.vol = vol;
   b.use_tile = any && vol <= cap;
   return b;
 }
 
-// Fill the shared gather box (float4 per node, box-local order) with value(idx) for every
-// node idx of the box, one node per thread.  Called right after box_extent (whose barrier
-// separates it from earlier readers of the box); synchronises after.
-template <int D, typename Value>
-__device__ __forceinline__ void box_load(const BoxInfo<D>& b, float4* sm4, Value&& value) {
-  if (b.use_tile)
-    for (int l = threadIdx.x; l < b.vol; l += blockDim.x) {
-      int idx[D], r = l;
+// Fill the shared gather box (float4 per node, box-local order), one node per thread: raw(f)
+// reads what node f of the scene's grid needs, value(raw, wall) turns it into the gathered
+// quantity.  BATCH nodes a thread are read before the first is used, so the box of a tile
+// costs one round trip to the L2.  Called right after box_extent (whose barrier separates it
+// from earlier readers of the box); synchronises after.
+template <int D, int BATCH, typename Raw, typename Value>
+__device__ __forceinline__ void box_load(const BoxInfo<D>& b, float4* sm4, const SimParams& P, Raw&& raw,
+                                         Value&& value) {
+  if (b.use_tile) {
+    // box-local index -> node by float reciprocals: with q the quotient and d the divisor, the
+    // quotient's error is below 3e-7 q and its distance to the next integer at least 0.5 / d,
+    // so the truncation is exact while q d < 1.6e6 (a box holds at most 12,288 nodes)
+    const float rz = __fdividef(1.0f, (float)b.dim[D - 1]), ry = D == 3 ? __fdividef(1.0f, (float)b.dim[1]) : 0.0f;
+#pragma unroll 1
+    for (int l0 = threadIdx.x; l0 < b.vol; l0 += BATCH * kTile) {
+      decltype(raw(0)) r[BATCH];
+      bool wall[BATCH];
 #pragma unroll
-      for (int a = D - 1; a >= 0; --a) {
-        idx[a] = b.lo[a] + r % b.dim[a];
-        r /= b.dim[a];
+      for (int u = 0; u < BATCH; ++u) {
+        const int l = l0 + u * kTile;
+        if (l < b.vol) {
+          int idx[D];
+          int q = (int)(((float)l + 0.5f) * rz);
+          idx[D - 1] = b.lo[D - 1] + (l - q * b.dim[D - 1]);
+          if (D == 3) {
+            const int x = (int)(((float)q + 0.5f) * ry);
+            idx[1] = b.lo[1] + (q - x * b.dim[1]);
+            q = x;
+          }
+          idx[0] = b.lo[0] + q;
+          wall[u] = is_wall<D>(idx, P);
+          r[u] = raw(node_flat<D>(idx, P.n_grid));
+        }
       }
-      sm4[l] = value(idx);
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u)
+        if (l0 + u * kTile < b.vol) sm4[l0 + u * kTile] = value(r[u], wall[u]);
     }
+  }
   __syncthreads();
 }
 
 // Run body(load) with load(i, j, k) returning value(base + (i, j, k)): from the shared
 // gather box when it holds the CTA's stencils, else computed from global memory.
-template <int D, typename Value, typename Body>
-__device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm4, const int base[D],
-                                           Value&& value, Body&& body) {
+template <int D, typename Raw, typename Value, typename Body>
+__device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm4, const int base[D], const SimParams& P,
+                                           Raw&& raw, Value&& value, Body&& body) {
   if (b.use_tile) {
     int lb = base[0] - b.lo[0];
 #pragma unroll
@@ -369,7 +409,7 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
       idx[0] = base[0] + i;
       idx[1] = base[1] + j;
       if (D == 3) idx[D - 1] = base[D - 1] + k;
-      return value(idx);
+      return value(raw(node_flat<D>(idx, P.n_grid)), is_wall<D>(idx, P));
     });
   }
 }
@@ -404,18 +444,17 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
 template <int D>
 __device__ __forceinline__ void put_record(float4* rec, bool valid, const Axes<D>& s, const float a[D],
                                            const float B[D][D], float dx) {
-  float ac[D], Bd[D][D], w[D][3];
+  float ac[D], Bd[D][D];
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    ac[c] = valid ? a[c] : 0.0f;
+    ac[c] = a[c];
 #pragma unroll
     for (int b = 0; b < D; ++b) {
-      Bd[c][b] = valid ? B[c][b] * dx : 0.0f;
+      Bd[c][b] = B[c][b] * dx;
       ac[c] += Bd[c][b] * (1.0f - s.f[b]);
     }
-#pragma unroll
-    for (int o = 0; o < 3; ++o) w[c][o] = valid ? s.w[c][o] : 0.0f;
   }
+  const float (&w)[D][3] = s.w;
   const float base = __int_as_float(valid ? pack_base<D>(s.base) : -1);
   float4* r = rec + threadIdx.x;
   r[0] = make_float4(w[0][0], w[0][1], w[0][2], 0.0f);
@@ -489,11 +528,13 @@ struct NodeSum<D, WITH_MASS, true> {
   }
 };
 
-// Scatter the warp's 32 records (written by its own lanes, __syncwarp'ed) into grid g.
+// Scatter the warp's 32 records (written by its own lanes, __syncwarp'ed) into grid g.  Slots: three
+// of nine columns in 3D (27 lanes, 10 or 11 particles each), eight of three in 2D (24 lanes, four
+// particles each, so that the slots' moves fall on the same turns).
 template <int D, bool WITH_MASS, bool DET>
 __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n, float mass_c, float fix0,
                                              float fix1, unsigned& err) {
-  constexpr int COLS = D == 3 ? 9 : 3, SLOTS = 32 / COLS;
+  constexpr int COLS = D == 3 ? 9 : 3, SLOTS = D == 3 ? 3 : 8;
   const int lane = threadIdx.x & 31;
   const int slot = lane / COLS, col = lane - slot * COLS;
   if (slot >= SLOTS) return;
@@ -510,8 +551,7 @@ __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n
 #pragma unroll 1
   for (; r < end; ++r) {
     const float* w0 = reinterpret_cast<const float*>(r);
-    float wz[3], qc[D], Bz[D];  // weights along the last axis; value at the column's centre; its increment
-    float wc;
+    float wc, wz[3], qc[D], Bz[D];  // weight of the column, along the last axis; value at its centre, increment
     int base;
     if (D == 3) {
       const float4 q2 = r[2 * kTile], q3 = r[3 * kTile], q4 = r[4 * kTile], q5 = r[5 * kTile];
@@ -539,9 +579,10 @@ __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n
       Bz[0] = q2.w;
       Bz[1] = q3.y;
     }
-    if (base != cur && base >= 0) {
+    if (base != cur) {
+      if (base < 0) continue;  // no scatter
       // base and cur hold the last axis in their low bits and differ by at least 3 across rows
-      // (the last axis stays below its field's range), so a small difference is a move along it
+      // (the last axis stays below its field's range), so a difference of one is a move along it
       const int d = base - cur;
       if (cur >= 0 && d == 1) {
         a0.reduce(g, node, mass_c);
@@ -559,12 +600,8 @@ __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n
         if (cur >= 0) {
           a0.reduce(g, node, mass_c);
           a1.reduce(g, node + 1, mass_c);
-          if (d == 2) {
-            a0 = a2;
-          } else {
-            a2.reduce(g, node + 2, mass_c);
-            a0.zero();
-          }
+          a2.reduce(g, node + 2, mass_c);
+          a0.zero();
           a1.zero();
           a2.zero();
         }
@@ -619,22 +656,14 @@ __device__ __forceinline__ void load_E(const float* rows, int64_t N, int64_t p, 
 // ---------------------------------------------------------------------------
 // grid functions applied at gather time
 // ---------------------------------------------------------------------------
-template <int D>
-__device__ __forceinline__ bool is_wall(const int idx[D], const SimParams& P) {
-  bool wall = false;
-#pragma unroll
-  for (int a = 0; a < D; ++a) wall = wall || idx[a] < P.wall || idx[a] >= P.n_grid - P.wall;
-  return wall;
-}
-
 // grid_op: v = p/m + dt g for m > 0 off the sticky walls, else 0 (w keeps m).  Rounding is
 // spelled out (no compiler-chosen contraction), so a node gives the same bits whether it
 // is staged in the shared gather box or read directly.
 template <int D>
-__device__ __forceinline__ float4 node_velocity(float4 pm, const int idx[D], const SimParams& P) {
+__device__ __forceinline__ float4 node_velocity(float4 pm, bool wall, const SimParams& P) {
   float4 u = make_float4(0.0f, 0.0f, 0.0f, pm.x);
-  if (pm.x > 0.0f && !is_wall<D>(idx, P)) {
-    const float im = __fdiv_rn(1.0f, pm.x);
+  if (pm.x > 0.0f && !wall) {
+    const float im = __frcp_rn(pm.x);
     u.x = __fmaf_rn(pm.y, im, __fmul_rn(P.dt, P.gravity[0]));
     u.y = __fmaf_rn(pm.z, im, __fmul_rn(P.dt, P.gravity[1]));
     if (D == 3) u.z = __fmaf_rn(pm.w, im, __fmul_rn(P.dt, P.gravity[2]));
@@ -645,11 +674,10 @@ __device__ __forceinline__ float4 node_velocity(float4 pm, const int idx[D], con
 // grid_op.grad: pbar = ubar / m and mbar = -ubar . (p / m) / m for m > 0 off the walls
 // (rounding spelled out as in node_velocity)
 template <int D>
-__device__ __forceinline__ float4 node_adjoint(float4 ub, float4 pm, const int idx[D],
-                                               const SimParams& P) {
+__device__ __forceinline__ float4 node_adjoint(float4 ub, float4 pm, bool wall, const SimParams& P) {
   float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (pm.x > 0.0f && !is_wall<D>(idx, P)) {
-    const float im = __fdiv_rn(1.0f, pm.x);
+  if (pm.x > 0.0f && !wall) {
+    const float im = __frcp_rn(pm.x);
     r.x = __fmul_rn(ub.x, im);
     r.y = __fmul_rn(ub.y, im);
     float dot = __fmaf_rn(ub.y, pm.z, __fmul_rn(ub.x, pm.y));
@@ -665,11 +693,21 @@ __device__ __forceinline__ float4 node_adjoint(float4 ub, float4 pm, const int i
 // ---------------------------------------------------------------------------
 // clears and box resets (each CTA takes its share of its own scene)
 // ---------------------------------------------------------------------------
+// The boxes of the jobs are copied to shared memory at the start of a tile (stage_clears:
+// asynchronous, 8 threads a job) and the clears run after a later barrier, off the chain of loads that
+// the tile starts with.
+__device__ __forceinline__ void stage_clears(const Clears& C, int scene, int* boxes) {
+  if ((int)threadIdx.x < 8 * C.n) {
+    const int* src = C.job[threadIdx.x >> 3].box + scene * 8 + (threadIdx.x & 7);
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(boxes + threadIdx.x);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+  }
+}
 template <int D>
-__device__ __forceinline__ void run_clears(const Clears& C, int scene, int rank, int nranks,
+__device__ __forceinline__ void run_clears(const Clears& C, const int* boxes, int scene, int rank, int nranks,
                                            int nnodes, int n) {
   for (int c = 0; c < C.n; ++c) {
-    const int* bb = C.job[c].box + scene * 8;
+    const int* bb = boxes + 8 * c;
     // An empty box (lo = INT_MAX, hi = INT_MIN: a buffer that was allocated but never
     // scattered into, e.g. after a pass that gave up) clears nothing; hi - lo is formed
     // only for a non-empty box, and the box is clipped to the grid.
@@ -704,15 +742,15 @@ __device__ __forceinline__ void reset_box(int* box, int scene) {
 // ---------------------------------------------------------------------------
 // P2G of the CTA's particles: stress, affine matrix A = kappa tau + m C, scatter
 // (m, m v + A dpos) into the scene grid g, fold the touched box into box_scene.
-// Every thread calls it; s_bbox must have been reset before an earlier barrier.
+// Every thread calls it; wb has not been used since an earlier barrier.
 // ---------------------------------------------------------------------------
 template <int D, int MAT, bool DET>
 __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis, bool active, int scene,
                                          int64_t p, const float x[D], const float v[D],
                                          const float C[D][D], const float E[D][D], float mu_p,
                                          float la_p, int mat_p, const int* group, const float* wact,
-                                         float4* g, int* box_scene, float4* rec, int* s_bbox,
-                                         unsigned& err, const double* R_in, double* R_out, int64_t N) {
+                                         float4* g, int* box_scene, float4* rec, WarpBounds& wb,
+                                         int seen, unsigned& err, const double* R_in, double* R_out, int64_t N) {
   Axes<D> s;
   bool ok = make_axes<D>(x, P, s) && active;
   if (active && !ok) err |= kErrOOB;
@@ -744,25 +782,29 @@ __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis,
   }
   __syncwarp();  // the warp's records may still be read by its earlier scatter
   put_record<D>(rec, ok, s, mv, Am, P.dx);
-  warp_bbox<D>(ok, s.base, s_bbox);
+  warp_bounds<D>(ok, s.base, wb);
   __syncwarp();
   scatter_runs<D, true, DET>(rec, g, P.n_grid, P.p_mass, P.fix_m, P.fix_p, err);
   __syncthreads();  // every warp's share of the box
-  cta_bbox_flush<D>(s_bbox, box_scene);
+  cta_bbox_flush<D>(wb, box_scene, seen);
 }
 
 // ---------------------------------------------------------------------------
 // forward particle pass: [G2P of step t-1] then [P2G of step t]
 // ---------------------------------------------------------------------------
 // One tile of a forward pass; every thread of the CTA calls it.  sm: dynamic shared memory
-// (step_smem_bytes), s_box: 8 * kBoxSlots ints, s_bbox: 8 ints.  A CTA that runs several tiles must
-// synchronise between them.
+// (step_smem_bytes).  A CTA that runs several tiles must synchronise between them.
+//
+// A tile is a chain of dependent round trips to the L2 -- its entry, its particles' rows, its
+// box of grid nodes -- and a 2,048-tile cube runs in two waves of 7 tiles per SM, so what is
+// not part of the chain stays off it: the clear jobs' boxes, mu and la come by asynchronous
+// copies, the bounds of a box need one barrier and no reset, all nodes of a box are read
+// before the first is used, and a warp scatters without waiting for the others.
 template <int D, int MAT, int MODE, bool NC, bool DET>
 __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A, int tile_index,
-                                          float* sm, int* s_box, int* s_bbox) {
+                                          float* sm, TileShared& sh) {
   using R = Rows<D>;
-  cta_bbox_reset(s_bbox);
-  reset_box_slots(s_box);
+  constexpr int kBatch = 3;
   float4* rec = reinterpret_cast<float4*>(sm + box_floats(P.gather_capacity));
   const int4 tile = A.tiles[tile_index];
   const int scene = tile.x;
@@ -771,7 +813,20 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
   const int64_t N = A.N;
   const int n = P.n_grid;
   unsigned err = 0;
-  run_clears<D>(A.clears, scene, tile.w, A.scene_tiles[scene], P.nnodes, n);
+  const int seen = MODE != kG2POnlyFull ? box_seen(A.box_w + scene * 8) : 0;
+  // the particle's rows first: in flight while the clears below read their boxes
+  float x[D], v[D], C[D][D], E[D][D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    x[a] = A.in[(R::X + a) * N + p];
+    if (MODE == kP2GOnly) v[a] = A.in[(R::V + a) * N + p];
+  }
+  if (MODE == kP2GOnly)
+#pragma unroll
+    for (int i = 0; i < D * D; ++i) C[i / D][i % D] = A.in[(R::C + i) * N + p];
+  load_E<D>(A.in, N, p, P.f_diag, E);
+  const int nranks = A.scene_tiles[scene];
+  stage_clears(A.clears, scene, sh.clear_box);
   if (tile.w == 0) reset_box(A.box_reset, scene);
   float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
   if (MODE != kG2POnlyFull) {
@@ -779,25 +834,15 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     stage_row(stage, 1, A.la + p);
   }
   stage_commit();
-  __syncthreads();  // s_bbox reset
 
-  float x[D], v[D], C[D][D], E[D][D];
-  if (MODE == kP2GOnly) {
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      x[a] = A.in[(R::X + a) * N + p];
-      v[a] = A.in[(R::V + a) * N + p];
-    }
-#pragma unroll
-    for (int i = 0; i < D * D; ++i) C[i / D][i % D] = A.in[(R::C + i) * N + p];
-    load_E<D>(A.in, N, p, P.f_diag, E);
-  } else {
+  if (MODE != kP2GOnly) {
     // ---- G2P: v' = sum W u, C' = 4/dx^2 sum W (u - u_c) dpos^T, x' = x + dt v',
     //      E' = E + dt C' (I + E), with u = grid_op(PM of step t-1) at each node
     float xo[D], Eo[D][D];
 #pragma unroll
-    for (int a = 0; a < D; ++a) xo[a] = A.in[(R::X + a) * N + p];
-    load_E<D>(A.in, N, p, P.f_diag, Eo);
+    for (int a = 0; a < D; ++a) xo[a] = x[a];
+#pragma unroll
+    for (int i = 0; i < D * D; ++i) Eo[i / D][i % D] = E[i / D][i % D];
     Axes<D> s;
     const bool ok = make_axes<D>(xo, P, s) && active;
     if (active && !ok) err |= kErrOOB;
@@ -809,35 +854,79 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
       for (int b = 0; b < D; ++b) B[a][b] = 0.0f;
     }
     const float4* PMg = scene_grid(A.PMr, scene, P);
-    auto velocity = [&](const int idx[D]) { return node_velocity<D>(pm_load<NC, DET>(PMg, node_flat<D>(idx, n), P), idx, P); };
+    stage_wait<0>();  // (this thread's share of the clear boxes, before the barrier below)
+    auto raw = [&](int f) { return pm_load<NC, DET>(PMg, f, P); };
+    auto velocity = [&](float4 pm, bool wall) { return node_velocity<D>(pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
     if (P.gather_capacity > 0) {
-      gbx = box_extent<D>(ok, s.base, P.gather_capacity, s_box);  // slot 0
+      gbx = box_extent<D>(ok, s.base, P.gather_capacity, sh.gather[0]);
       if (A.box_stats && threadIdx.x == 0 && gbx.vol > 0) {
         atomicAdd(A.box_stats, 1ull);
         if (!gbx.use_tile) atomicAdd(A.box_stats + 1, 1ull);
       }
-      box_load<D>(gbx, reinterpret_cast<float4*>(sm), velocity);
+      box_load<D, kBatch>(gbx, reinterpret_cast<float4*>(sm), P, raw, velocity);
+    } else {
+      __syncthreads();
     }
+    run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
     if (ok) {
       // centred on the stencil's centre node: equal because sum W dpos = 0, and
       // accurate in FP32 when u is nearly uniform over the stencil
-      with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, velocity, [&](auto load) {
+      with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, P, raw, velocity, [&](auto load) {
         const float4 uc4 = load(1, 1, D == 3 ? 1 : 0);
         const float uc[3] = {uc4.x, uc4.y, uc4.z};
-        for_nodes<D>(s.w, [&](int i, int j, int k, float W) {
-          const float4 u4 = load(i, j, k);
-          const float u[3] = {u4.x, u4.y, u4.z};
-          const float dpos[3] = {s.dp[0][i], s.dp[1][j], D == 3 ? s.dp[D - 1][k] : 0.0f};
+        GatherAxes<D> g(s);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          float wi, dwi, dpi, t[D], tb[D][D];  // sums over the plane: W d, and W d dpos_b (b >= 1)
+          axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
 #pragma unroll
           for (int a = 0; a < D; ++a) {
-            v[a] += W * u[a];
-            const float wd = W * (u[a] - uc[a]);
+            t[a] = 0.0f;
 #pragma unroll
-            for (int b = 0; b < D; ++b) B[a][b] += wd * dpos[b];
+            for (int b = 1; b < D; ++b) tb[a][b] = 0.0f;
           }
-        });
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            float r[D], rb[D];  // the same along the last axis
+            if (D == 3) {
+#pragma unroll
+              for (int a = 0; a < D; ++a) r[a] = rb[a] = 0.0f;
+#pragma unroll
+              for (int k = 0; k < 3; ++k) {
+                const float4 u4 = load(i, j, k);
+                const float u[3] = {u4.x, u4.y, u4.z};
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                  const float d = u[a] - uc[a];
+                  r[a] += s.w[D - 1][k] * d;
+                  rb[a] += g.wp[D - 1][k] * d;
+                }
+              }
+            } else {
+              const float4 u4 = load(i, j, 0);
+              r[0] = u4.x - uc[0];
+              r[1] = u4.y - uc[1];
+            }
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+              t[a] += s.w[1][j] * r[a];
+              tb[a][1] += g.wp[1][j] * r[a];
+              if (D == 3) tb[a][D - 1] += s.w[1][j] * rb[a];
+            }
+          }
+          const float wpi = wi * dpi;
+#pragma unroll
+          for (int a = 0; a < D; ++a) {
+            v[a] += wi * t[a];
+            B[a][0] += wpi * t[a];
+#pragma unroll
+            for (int b = 1; b < D; ++b) B[a][b] += wi * tb[a][b];
+          }
+        }
+#pragma unroll
+        for (int a = 0; a < D; ++a) v[a] += uc[a];  // sum W = 1
       });
     }
     const float c4 = 4.0f * P.inv_dx * P.inv_dx;
@@ -875,11 +964,17 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     stage_wait<0>();
     p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, x, v, C, E, staged(stage, 0), staged(stage, 1),
                           MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact, scene_grid(A.PMw, scene, P),
-                          A.box_w + scene * 8, rec, s_bbox, err, nullptr, A.Rw, N);
+                          A.box_w + scene * 8, rec, sh.scatter[0], seen, err, nullptr, A.Rw, N);
+    if (MODE == kP2GOnly) run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
   }
   if (err) atomicOr(A.err, err);
 }
 
+// resident CTAs per SM the adjoint passes are compiled for
+template <int D>
+constexpr int adj_ctas_per_sm() {
+  return D == 2 ? MPM_ADJ_CTAS_PER_SM_2D : MPM_ADJ_CTAS_PER_SM_3D;
+}
 // resident CTAs per SM the forward passes are compiled for
 template <int D, int MAT>
 constexpr int step_ctas_per_sm() {
@@ -892,9 +987,8 @@ template <int D, int MAT, int MODE, bool DET>
 __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
     step_kernel(const __grid_constant__ SimParams P, const __grid_constant__ StepArgs A) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ int s_box[8 * kBoxSlots];
-  __shared__ int s_bbox[8];
-  step_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox);
+  __shared__ TileShared sh;
+  step_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -904,12 +998,9 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
 // One tile of an adjoint pass (same calling rules as step_tile; s_wbar: kWbarSlots floats).
 template <int D, int MAT, int MODE, bool NC, bool DET>
 __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& A, int tile_index,
-                                             float* sm, int* s_box, int* s_bbox_ub, int* s_bbox_pm,
-                                             float* s_wbar) {
+                                             float* sm, TileShared& sh, float* s_wbar) {
   using R = Rows<D>;
-  cta_bbox_reset(s_bbox_ub);
-  cta_bbox_reset(s_bbox_pm);
-  reset_box_slots(s_box);
+  constexpr int kBatch = 3;
   float4* rec = reinterpret_cast<float4*>(sm + box_floats(P.gather_capacity));
   const int4 tile = A.tiles[tile_index];
   const int scene = tile.x;
@@ -919,12 +1010,15 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   const int n = P.n_grid;
   const float c4 = 4.0f * P.inv_dx * P.inv_dx;
   unsigned err = 0;
-  run_clears<D>(A.clears, scene, tile.w, A.scene_tiles[scene], P.nnodes, n);
+  const int seen_ub = MODE != kAdjP2G && A.box_ub ? box_seen(A.box_ub + scene * 8) : 0;
+  const int seen_m = MODE != kAdjP2G && A.stm ? box_seen(A.box_m + scene * 8) : 0;
+  const int nranks = A.scene_tiles[scene];
+  stage_clears(A.clears, scene, sh.clear_box);
+  stage_commit();
   if (tile.w == 0) {
     reset_box(A.box_ub_reset, scene);
     reset_box(A.box_m_reset, scene);
   }
-  __syncthreads();  // shared boxes reset
   // stage what the G2P-adjoint (state s: x, F) and the recomputed P2G (state s-1, mu, la)
   // read, so that those loads are in flight during the P2G-adjoint
   float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
@@ -1010,65 +1104,91 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
     const float4* UBg = scene_grid(A.UB1, scene, P);
     const float4* PMg = scene_grid(A.PM1, scene, P);
-    auto pbar = [&](const int idx[D]) {
-      const int f = node_flat<D>(idx, n);
-      return node_adjoint<D>(ub_load<NC, DET>(UBg, f, P, A.ub_m0), pm_load<NC, DET>(PMg, f, P), idx, P);
-    };
+    auto raw = [&](int f) { return NodePair{ub_load<NC, DET>(UBg, f, P, A.ub_m0), pm_load<NC, DET>(PMg, f, P)}; };
+    auto pbar = [&](const NodePair& g, bool wall) { return node_adjoint<D>(g.ub, g.pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
+    stage_wait<2>();  // this thread's share of the clear boxes, before the barrier below
     if (P.gather_capacity > 0) {
-      gbx = box_extent<D>(ok, s.base, P.gather_capacity, s_box);  // slot 0
-      box_load<D>(gbx, reinterpret_cast<float4*>(sm), pbar);
+      gbx = box_extent<D>(ok, s.base, P.gather_capacity, sh.gather[0]);
+      box_load<D, 2>(gbx, reinterpret_cast<float4*>(sm), P, raw, pbar);
+    } else {
+      __syncthreads();
     }
-    if (ok) with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, pbar, [&](auto load) {
+    run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
+    if (ok) with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, P, raw, pbar, [&](auto load) {
       // pbar - pbar_c and mbar - mbar_c (centre node) in the moment and weight-gradient
       // terms: equal to the plain sums because sum W dpos = 0, sum grad W = 0 and
       // sum grad W dpos^T = I, without the FP32 cancellation of a smooth pbar field
       const float4 gc = load(1, 1, D == 3 ? 1 : 0);
       const float pc[3] = {gc.x, gc.y, gc.z};
-#pragma unroll
+      GatherAxes<D> ga(s);
+#pragma unroll(D == 3 ? 1 : 3)
       for (int i = 0; i < 3; ++i) {
-        float qi[D];
+        float wi, dwi, dpi, qi[D], t[D], tb[D][D], e[D];
+        axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
 #pragma unroll
-        for (int c = 0; c < D; ++c) qi[c] = mv[c] + Am[c][0] * s.dp[0][i];
+        for (int c = 0; c < D; ++c) {
+          qi[c] = mv[c] + Am[c][0] * dpi;
+          t[c] = e[c] = 0.0f;  // e[b]: sum of W-bar times the weight, differentiated along b >= 1
+#pragma unroll
+          for (int b = 1; b < D; ++b) tb[c][b] = 0.0f;
+        }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          const float wij = s.w[0][i] * s.w[1][j];
-          const float dwij0 = s.dw[0][i] * s.w[1][j];
-          const float dwij1 = s.w[0][i] * s.dw[1][j];
-          float qij[D];
+          float qij[D], r[D], rb[D], e0 = 0.0f, e1 = 0.0f;
 #pragma unroll
-          for (int c = 0; c < D; ++c) qij[c] = qi[c] + Am[c][1] * s.dp[1][j];
+          for (int c = 0; c < D; ++c) {
+            qij[c] = qi[c] + Am[c][1] * s.dp[1][j];
+            r[c] = rb[c] = 0.0f;
+          }
 #pragma unroll
           for (int k = 0; k < (D == 3 ? 3 : 1); ++k) {
-            const float wk = D == 3 ? s.w[D - 1][k] : 1.0f;
-            const float W = wij * wk;
-            float gW[D];
-            gW[0] = dwij0 * wk;
-            gW[1] = dwij1 * wk;
-            if (D == 3) gW[D - 1] = wij * s.dw[D - 1][k];
-            float q[D];
-#pragma unroll
-            for (int c = 0; c < D; ++c)
-              q[c] = D == 3 ? qij[c] + Am[c][D - 1] * s.dp[D - 1][k] : qij[c];
-            const float dpos[3] = {s.dp[0][i], s.dp[1][j], D == 3 ? s.dp[D - 1][k] : 0.0f};
             const float4 g4 = load(i, j, k);
             const float pb[3] = {g4.x, g4.y, g4.z};
             float Wbar = P.p_mass * (g4.w - gc.w);
 #pragma unroll
             for (int c = 0; c < D; ++c) {
-              const float dpb = pb[c] - pc[c];
-              Wbar += dpb * q[c];
-              vb[c] += W * pb[c];
-              sw[c] += W * dpb;
-#pragma unroll
-              for (int b = 0; b < D; ++b) Ab[c][b] += W * dpb * dpos[b];
+              const float d = pb[c] - pc[c];
+              Wbar += d * (D == 3 ? qij[c] + Am[c][D - 1] * s.dp[D - 1][k] : qij[c]);
+              if (D == 3) {
+                r[c] += s.w[D - 1][k] * d;
+                rb[c] += ga.wp[D - 1][k] * d;
+              } else {
+                r[c] = d;
+              }
             }
-#pragma unroll
-            for (int b = 0; b < D; ++b) xg[b] += Wbar * gW[b];
+            if (D == 3) {
+              e0 += s.w[D - 1][k] * Wbar;
+              e1 += s.dw[D - 1][k] * Wbar;
+            } else {
+              e0 = Wbar;
+            }
           }
+#pragma unroll
+          for (int c = 0; c < D; ++c) {
+            t[c] += s.w[1][j] * r[c];
+            tb[c][1] += ga.wp[1][j] * r[c];
+            if (D == 3) tb[c][D - 1] += s.w[1][j] * rb[c];
+          }
+          e[0] += s.w[1][j] * e0;
+          e[1] += s.dw[1][j] * e0;
+          if (D == 3) e[D - 1] += s.w[1][j] * e1;
         }
+        const float wpi = wi * dpi;
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          sw[c] += wi * t[c];
+          Ab[c][0] += wpi * t[c];
+#pragma unroll
+          for (int b = 1; b < D; ++b) Ab[c][b] += wi * tb[c][b];
+        }
+        xg[0] += dwi * e[0];
+#pragma unroll
+        for (int b = 1; b < D; ++b) xg[b] += wi * e[b];
       }
+#pragma unroll
+      for (int c = 0; c < D; ++c) vb[c] = pc[c] + sw[c];  // sum W = 1
     });
     if (kLate) load_carried();
     // x += inv_dx sum Wbar gradW - A^T sum W dpbar
@@ -1154,7 +1274,6 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   // ---- G2P adjoint of step s: x' = x + dt v', E' = E + dt C' (I + E) ----
   {
     float x0[D], E0[D][D];
-#pragma unroll
     stage_wait<0>();
 #pragma unroll
     for (int a = 0; a < D; ++a) x0[a] = staged(stage, a);
@@ -1204,55 +1323,75 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(bound));
       if ((threadIdx.x & 31) == 0 && mb != 0u) atomicMax(A.ub_m0, mb);
       if (err) atomicOr(A.err, err);
+      __syncthreads();
+      run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
       return;
     }
     const float4* PMg = scene_grid(A.PM0, scene, P);
-    auto velocity = [&](const int idx[D]) { return node_velocity<D>(pm_load<NC, DET>(PMg, node_flat<D>(idx, n), P), idx, P); };
+    auto raw = [&](int f) { return pm_load<NC, DET>(PMg, f, P); };
+    auto velocity = [&](float4 pm, bool wall) { return node_velocity<D>(pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
-    if (P.gather_capacity > 0) gbx = box_extent<D>(ok, s.base, P.gather_capacity, s_box + 8);  // slot 1
-    if (P.gather_capacity > 0) box_load<D>(gbx, reinterpret_cast<float4*>(sm), velocity);
-    if (ok) with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, velocity, [&](auto load) {
+    if (P.gather_capacity > 0) {
+      gbx = box_extent<D>(ok, s.base, P.gather_capacity, sh.gather[1]);
+      box_load<D, kBatch>(gbx, reinterpret_cast<float4*>(sm), P, raw, velocity);
+    } else if (MODE == kAdjG2P) {
+      __syncthreads();
+    }
+    if (MODE == kAdjG2P) run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
+    if (ok) with_nodes<D>(gbx, reinterpret_cast<const float4*>(sm), s.base, P, raw, velocity, [&](auto load) {
       // x-adjoint terms on u - u_c (centre node), by the same B-spline identities
       const float4 uc4 = load(1, 1, D == 3 ? 1 : 0);
       const float uc[3] = {uc4.x, uc4.y, uc4.z};
       float xg[D], sw[D];
 #pragma unroll
       for (int a = 0; a < D; ++a) xg[a] = sw[a] = 0.0f;
-#pragma unroll
+#pragma unroll(D == 3 ? 1 : 3)
       for (int i = 0; i < 3; ++i) {
-        float qi[D];
+        float wi, dwi, dpi, qi[D], t[D], e[D];
+        axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
 #pragma unroll
-        for (int c = 0; c < D; ++c) qi[c] = vt[c] + c4 * Ct[c][0] * s.dp[0][i];
+        for (int c = 0; c < D; ++c) {
+          qi[c] = vt[c] + c4 * Ct[c][0] * dpi;
+          t[c] = e[c] = 0.0f;
+        }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          const float wij = s.w[0][i] * s.w[1][j];
-          const float dwij0 = s.dw[0][i] * s.w[1][j];
-          const float dwij1 = s.w[0][i] * s.dw[1][j];
-          float qij[D];
+          float qij[D], r[D], e0 = 0.0f, e1 = 0.0f;
 #pragma unroll
-          for (int c = 0; c < D; ++c) qij[c] = qi[c] + c4 * Ct[c][1] * s.dp[1][j];
+          for (int c = 0; c < D; ++c) {
+            qij[c] = qi[c] + c4 * Ct[c][1] * s.dp[1][j];
+            r[c] = 0.0f;
+          }
 #pragma unroll
           for (int k = 0; k < (D == 3 ? 3 : 1); ++k) {
-            const float wk = D == 3 ? s.w[D - 1][k] : 1.0f;
-            const float W = wij * wk;
-            float gW[D];
-            gW[0] = dwij0 * wk;
-            gW[1] = dwij1 * wk;
-            if (D == 3) gW[D - 1] = wij * s.dw[D - 1][k];
             const float4 u4 = load(i, j, k);
-            const float du[3] = {u4.x - uc[0], u4.y - uc[1], u4.z - uc[2]};
+            const float u[3] = {u4.x, u4.y, u4.z};
             float Wbar = 0.0f;
 #pragma unroll
             for (int c = 0; c < D; ++c) {
-              const float q = D == 3 ? qij[c] + c4 * Ct[c][D - 1] * s.dp[D - 1][k] : qij[c];
-              Wbar += du[c] * q;
-              sw[c] += W * du[c];
+              const float d = u[c] - uc[c];
+              Wbar += d * (D == 3 ? qij[c] + c4 * Ct[c][D - 1] * s.dp[D - 1][k] : qij[c]);
+              r[c] = D == 3 ? r[c] + s.w[D - 1][k] * d : d;
             }
-#pragma unroll
-            for (int b = 0; b < D; ++b) xg[b] += Wbar * gW[b];
+            if (D == 3) {
+              e0 += s.w[D - 1][k] * Wbar;
+              e1 += s.dw[D - 1][k] * Wbar;
+            } else {
+              e0 = Wbar;
+            }
           }
+#pragma unroll
+          for (int c = 0; c < D; ++c) t[c] += s.w[1][j] * r[c];
+          e[0] += s.w[1][j] * e0;
+          e[1] += s.dw[1][j] * e0;
+          if (D == 3) e[D - 1] += s.w[1][j] * e1;
         }
+#pragma unroll
+        for (int c = 0; c < D; ++c) sw[c] += wi * t[c];
+        xg[0] += dwi * e[0];
+#pragma unroll
+        for (int b = 1; b < D; ++b) xg[b] += wi * e[b];
       }
 #pragma unroll
       for (int b = 0; b < D; ++b) {
@@ -1278,11 +1417,11 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     float fix_u = 1.0f, unfix_u = 1.0f;
     if (DET) ub_scales(A.ub_m0, fix_u, unfix_u);
     put_record<D>(rec, ok, s, vt, Bs, P.dx);
-    warp_bbox<D>(ok, s.base, s_bbox_ub);
+    warp_bounds<D>(ok, s.base, sh.scatter[0]);
     __syncwarp();
     scatter_runs<D, false, DET>(rec, UBs, n, 0.0f, fix_u, fix_u, err);
     __syncthreads();  // every warp's share of the box
-    cta_bbox_flush<D>(s_bbox_ub, A.box_ub + scene * 8);
+    cta_bbox_flush<D>(sh.scatter[0], A.box_ub + scene * 8, seen_ub);
   }
 
   // ---- recomputed P2G of step s-1 (the grid of the next adjoint pass) ----
@@ -1303,21 +1442,20 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       for (int j = 0; j < D; ++j) E[i][j] = staged(stage, b + R::F + i * D + j) - (i == j ? P.f_diag : 0.0f);
     p2g_pass<D, MAT, DET>(P, P.basis2, active, scene, p, x, v, C, E, staged(stage, b + R::Q),
                           staged(stage, b + R::Q + 1), MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact,
-                          scene_grid(A.PMm, scene, P), A.box_m + scene * 8, rec, s_bbox_pm, err, A.Rm,
+                          scene_grid(A.PMm, scene, P), A.box_m + scene * 8, rec, sh.scatter[1],
+                          seen_m, err, A.Rm,
                           nullptr, N);
   }
   if (err) atomicOr(A.err, err);
 }
 
 template <int D, int MAT, int MODE, bool DET>
-__global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
+__global__ void __launch_bounds__(kTile, adj_ctas_per_sm<D>())
     adjoint_kernel(const __grid_constant__ SimParams P, const __grid_constant__ AdjArgs A) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ int s_box[8 * kBoxSlots];
-  __shared__ int s_bbox_ub[8];
-  __shared__ int s_bbox_pm[8];
+  __shared__ TileShared sh;
   __shared__ float s_wbar[kWbarSlots];
-  adjoint_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar);
+  adjoint_tile<D, MAT, MODE, true, DET>(P, A, blockIdx.x, sm, sh, s_wbar);
 }
 
 // ---------------------------------------------------------------------------
@@ -1428,8 +1566,7 @@ template <int D, int MAT, int MODE, bool DET>
 __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
     step_persistent_kernel(const PassEntry* plan, int n_pass, int n_tiles, PersistCtl ctl) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ int s_box[8 * kBoxSlots];
-  __shared__ int s_bbox[8];
+  __shared__ TileShared sh;
   __shared__ int s_go, s_tile;
   __shared__ PassEntry e;
   // a barrier of an earlier launch of this sequence gave up: its passes never finished, so
@@ -1440,7 +1577,7 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
     __syncthreads();
     cta_copy(&e, plan + i);
     for (int t; (t = next_tile(ctl, i, &s_tile)) < n_tiles;) {
-      step_tile<D, MAT, MODE, false, DET>(e.P, e.S, t, sm, s_box, s_bbox);
+      step_tile<D, MAT, MODE, false, DET>(e.P, e.S, t, sm, sh);
       __syncthreads();
     }
   }
@@ -1448,12 +1585,10 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
 
 // Adjoint-kind passes plan[0..n_pass), all of mode MODE.
 template <int D, int MAT, int MODE, bool DET>
-__global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
+__global__ void __launch_bounds__(kTile, adj_ctas_per_sm<D>())
     adjoint_persistent_kernel(const PassEntry* plan, int n_pass, int n_tiles, PersistCtl ctl) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ int s_box[8 * kBoxSlots];
-  __shared__ int s_bbox_ub[8];
-  __shared__ int s_bbox_pm[8];
+  __shared__ TileShared sh;
   __shared__ float s_wbar[kWbarSlots];
   __shared__ int s_go, s_tile;
   __shared__ PassEntry e;
@@ -1465,7 +1600,7 @@ __global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
     __syncthreads();
     cta_copy(&e, plan + i);
     for (int t; (t = next_tile(ctl, i, &s_tile)) < n_tiles;) {
-      adjoint_tile<D, MAT, MODE, false, DET>(e.P, e.A, t, sm, s_box, s_bbox_ub, s_bbox_pm, s_wbar);
+      adjoint_tile<D, MAT, MODE, false, DET>(e.P, e.A, t, sm, sh, s_wbar);
       __syncthreads();
     }
   }
@@ -1474,7 +1609,10 @@ __global__ void __launch_bounds__(kTile, MPM_ADJ_CTAS_PER_SM)
 // Zero the dirty boxes of the clear jobs (end of a launch sequence); blockIdx.y = scene.
 template <int D>
 __global__ void clear_kernel(const __grid_constant__ Clears C, int nnodes, int n) {
-  run_clears<D>(C, blockIdx.y, blockIdx.x, gridDim.x, nnodes, n);
+  __shared__ int boxes[8 * kMaxClears];
+  if ((int)threadIdx.x < 8 * C.n) boxes[threadIdx.x] = C.job[threadIdx.x >> 3].box[blockIdx.y * 8 + (threadIdx.x & 7)];
+  __syncthreads();
+  run_clears<D>(C, boxes, blockIdx.y, blockIdx.x, gridDim.x, nnodes, n);
 }
 
 }  // namespace mpm
