@@ -1,0 +1,76 @@
+"""Mass-spring systems whose springs reach every pair of masses (each pair is a branch of its own in
+the kernels), in either order of a spring's ends, for each kernel variant (at most 4 masses with
+springs unrolled or looped, up to 8 masses) and batch size (blocks of 128 and of 512 threads),
+against the FP64 oracle on sampled systems; a spring of zero length stays finite."""
+import itertools
+
+import numpy as np
+import pytest
+
+from mpm_testlib import rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ms():
+    from paper_1910_00935_gb300 import build, mass_spring
+    build.build()
+    return mass_spring
+
+
+def _springs(n, count, rng):
+    pairs = list(itertools.combinations(range(n), 2))
+    rng.shuffle(pairs)
+    return [tuple(p) if k % 2 else tuple(p[::-1]) for k, p in enumerate(pairs[:count])]
+
+
+@pytest.mark.parametrize("dim,n,count,S", [
+    (2, 1, 0, 5), (2, 2, 1, 1), (3, 3, 3, 129), (2, 4, 4, 300), (3, 4, 6, 301), (2, 8, 28, 200), (3, 8, 28, 77),
+    (3, 6, 3, 64), (2, 3, 3, 155648), (2, 3, 3, 155649), (3, 4, 5, 200003)])
+def test_every_pair_matches_oracle(ms, dim, n, count, S):
+    import oracle
+    rng = np.random.default_rng(100 * n + dim)
+    springs, T, k, alpha, dt, m = _springs(n, count, rng), 40, 60.0, 3.0, 2e-3, 1.2
+    base = rng.uniform(0.0, 0.3, (n, dim)) + 0.2 * np.arange(n)[:, None]
+    x0 = (base[None] + rng.normal(0, 0.01, (S, n, dim))).astype(np.float32)
+    v0 = rng.normal(0, 0.2, (S, n, dim)).astype(np.float32)
+    l0 = np.stack([np.linalg.norm(x0[:, a] - x0[:, b], axis=1) for a, b in springs], 1) if springs else np.zeros((S, 0))
+    l0 = (l0 * rng.uniform(0.8, 1.2, l0.shape)).astype(np.float32)
+    cx, cv = rng.normal(size=(2, S, n, dim)).astype(np.float32)
+    rows = lambda a: torch.as_tensor(np.ascontiguousarray(a.reshape(S, -1).T)).cuda()  # noqa: E731
+    sim = ms.MassSprings(dim, n, springs, S, k, alpha, dt, m, steps=T)
+    sim.forward(rows(x0), rows(v0), rows(l0) if springs else torch.zeros(1, S, device="cuda"), T)
+    xT, vT = sim.state()
+    gx, gv, gl = sim.backward(rows(cx), rows(cv))
+    sim.sync()
+    sim.close()
+    sample = sorted(set([0, S - 1] + list(rng.integers(0, S, 24))))
+    un = lambda t: t.cpu().numpy().T.astype(np.float64)[sample].reshape(len(sample), -1)  # noqa: E731
+    o = {key: [] for key in ("x", "v", "gx", "gv", "gl")}
+    for s in sample:
+        X, V = oracle.ms_forward(x0[s].astype(np.float64), v0[s].astype(np.float64), springs, l0[s].astype(np.float64), k, alpha,
+                                 float(np.float32(dt)), float(np.float32(m)), T)
+        a, b, c = oracle.ms_backward(X, springs, l0[s].astype(np.float64), k, alpha, float(np.float32(dt)), float(np.float32(m)),
+                                     cx[s].astype(np.float64), cv[s].astype(np.float64))
+        for key, val in zip(o, (X[-1], V[-1], a, b, c)):
+            o[key].append(np.ravel(val))
+    # the bars of the states' and gradients' parity tests
+    for key, got, tol in (("x", xT, 1e-5), ("v", vT, 1e-4), ("gx", gx, 1e-3), ("gv", gv, 1e-3), ("gl", gl, 1e-3)):
+        want = np.array(o[key])
+        if want.size:
+            assert rel_l2(un(got), want) <= tol, (key, rel_l2(un(got), want))
+
+
+def test_zero_length_spring_is_finite(ms):
+    """Two masses at one point: no force, no NaN, in both passes."""
+    x0 = torch.zeros(4, 3, device="cuda")
+    sim = ms.MassSprings(2, 2, [(0, 1)], 3, 50.0, 1.0, 1e-3, steps=5)
+    sim.forward(x0, torch.zeros_like(x0), torch.full((1, 3), 0.1, device="cuda"), 5)
+    x, v = sim.state()
+    gx, gv, gl = sim.backward(torch.ones_like(x0), None)
+    sim.sync()
+    sim.close()
+    assert float(x.abs().max()) == 0.0 and float(v.abs().max()) == 0.0
+    assert all(bool(torch.isfinite(t).all()) for t in (gx, gv, gl))
