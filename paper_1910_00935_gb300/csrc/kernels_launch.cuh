@@ -20,6 +20,22 @@ cudaError_t allow_smem(K k, size_t smem) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+// one CTA per tile; early: the pass may start while the one before it on the stream drains
+template <typename K, typename Args>
+cudaError_t launch_pass(K k, const SimParams& P, const Args& A, int n_tiles, size_t smem, cudaStream_t s, int early) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_tiles);
+  cfg.blockDim = dim3(kTile);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, P, A);
+}
+
 template <int D, int MAT, int MODE, bool DET>
 cudaError_t step_one(const SimParams& P, const StepArgs& A, int n_tiles, cudaStream_t s) {
   const size_t smem = step_smem_bytes<D>(P.gather_capacity);
@@ -33,8 +49,7 @@ cudaError_t step_one(const SimParams& P, const StepArgs& A, int n_tiles, cudaStr
     cudaFuncAttributes attr;
     return cudaFuncGetAttributes(&attr, k);
   }
-  k<<<n_tiles, kTile, smem, s>>>(P, A);
-  e = cudaGetLastError();
+  e = launch_pass(k, P, A, n_tiles, smem, s, A.early);
   if (e != cudaSuccess) note_launch_failure("step_kernel", D, MAT, MODE, smem, cudaSuccess);
   return e;
 }
@@ -52,8 +67,7 @@ cudaError_t adj_one(const SimParams& P, const AdjArgs& A, int n_tiles, cudaStrea
     cudaFuncAttributes attr;
     return cudaFuncGetAttributes(&attr, k);
   }
-  k<<<n_tiles, kTile, smem, s>>>(P, A);
-  e = cudaGetLastError();
+  e = launch_pass(k, P, A, n_tiles, smem, s, A.early);
   if (e != cudaSuccess) note_launch_failure("adjoint_kernel", D, MAT, MODE, smem, cudaSuccess);
   return e;
 }

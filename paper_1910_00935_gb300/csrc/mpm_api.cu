@@ -536,6 +536,11 @@ struct Launcher {
   cudaStream_t main_s = nullptr;  // (the caller's stream may be the legacy default, null)
   bool main_known = false;
   int pm_lo = 0, pm_hi = -1;
+  // whether the last operation issued on a stream (main, side) was a particle pass of this
+  // sequence: the next pass may then start while it drains (see pass_wait).  Anything else -- the
+  // sequence's start, a clear, an event to wait for, a controller kernel -- is waited for in full.
+  bool after_pass[2] = {false, false};
+  int sid() const { return h->pm.sid; }
 
   // issue on the main (0) or the side (1) stream from now on
   void use_stream(int sid) {
@@ -551,7 +556,10 @@ struct Launcher {
     pm_hi = pm_lo + h->m.pm_pool;
   }
   cudaError_t signal(cudaEvent_t ev) { return cudaEventRecord(ev, s); }
-  cudaError_t wait(cudaEvent_t ev) { return cudaStreamWaitEvent(s, ev, 0); }
+  cudaError_t wait(cudaEvent_t ev) {
+    after_pass[sid()] = false;
+    return cudaStreamWaitEvent(s, ev, 0);
+  }
 
   // clear, on the current stream, every buffer released on it and not yet cleared
   cudaError_t flush_clears() {
@@ -559,6 +567,7 @@ struct Launcher {
       Clears C = take_clears(h);
       if (C.n == 0) return cudaSuccess;
       ++count;
+      after_pass[sid()] = false;
       cudaError_t e = timed(MPM_KERNEL_GRID_CLEAR, [&] {
         return h->m.D == 2 ? launch_clear<2>(C, (int)h->m.nnodes, h->m.n_grid, h->m.S, grid_blocks_per_scene(h), s)
                            : launch_clear<3>(C, (int)h->m.nnodes, h->m.n_grid, h->m.S, grid_blocks_per_scene(h), s);
@@ -570,7 +579,7 @@ struct Launcher {
 
   // one pass: launched, recorded, or queued into the pending persistent run
   template <typename Args>
-  cudaError_t pass(int kind, int pmode, int category, const SimParams& P, const Args& A) {
+  cudaError_t pass(int kind, int pmode, int category, const SimParams& P, Args A) {
     if (mode == kRecord) {
       PassEntry e;
       memset(&e, 0, sizeof(e));
@@ -595,6 +604,8 @@ struct Launcher {
     }
     ++count;
     const Dims& m = h->m;
+    A.early = after_pass[sid()] && !h->profile;
+    after_pass[sid()] = true;
     return timed(category, [&] {
       if constexpr (std::is_same<Args, StepArgs>::value)
         return m.D == 2 ? launch_step<2>(h->desc.material, pmode, P, A, m.n_tiles, s)
@@ -769,6 +780,7 @@ struct Launcher {
     const Layout& L = h->L;
     const CtrlStep c = ctrl_step(h, t);
     count += 2;
+    after_pass[sid()] = false;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_forward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off), st,
                                  h->at<int>(L.group), h->at<double>(L.ctrl_part), h->at<float>(L.wact),
@@ -787,6 +799,7 @@ struct Launcher {
     const Layout& L = h->L;
     const CtrlStep c = ctrl_step(h, t);
     count += 2;
+    after_pass[sid()] = false;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_backward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off),
                                   h->at<int>(L.group), h->at<float>(L.wbar_tile), h->at<float>(L.wact),
