@@ -675,7 +675,7 @@ struct Launcher {
   // one forward particle pass: G2P of step t-1 from grid `read` (-1: none), P2G of step
   // t into a new grid (returned in *written, -1 for G2P only)
   cudaError_t step(int smode, int t, const float* in, float* out, int read, int* written,
-                   double* R_out = nullptr) {
+                   double* R_out = nullptr, bool sense = false) {
     const Dims& m = h->m;
     SimParams P = params_for(h, t);
     StepArgs A;
@@ -694,6 +694,7 @@ struct Launcher {
     A.box_stats = h->at<unsigned long long>(h->L.box_stats);
     if (read >= 0) A.PMr = ring_grid(h, h->pm, read);
     A.Rw = R_out;
+    if (sense) A.sense = h->at<float>(h->L.ctrl_part);
     if (written) {
       WriteSlot w;
       if (!ring_alloc(h, h->pm, w, pm_lo, pm_hi)) return cudaErrorMemoryAllocation;
@@ -716,7 +717,8 @@ struct Launcher {
   // when stm != null, the recomputed grid of step s-1 (*pm_written)
   cudaError_t adjoint(int amode, int s_step, const float* st1, const float* st0, const float* stm,
                       int pm1, int ub1, int pm0, int* ub_written, int* pm_written,
-                      const double* R1 = nullptr, const double* Rm = nullptr, int measure = 0) {
+                      const double* R1 = nullptr, const double* Rm = nullptr, int measure = 0,
+                      bool sense_add = false) {
     const Dims& m = h->m;
     SimParams P = params_for(h, s_step + 1);
     SimParams P2 = params_for(h, s_step - 1 >= 0 ? s_step - 1 : 0);
@@ -743,6 +745,7 @@ struct Launcher {
     A.Rm = Rm;
     A.ub_m0 = h->at<unsigned>(h->L.ub_m0);
     A.measure = measure;
+    if (sense_add) A.sense_add = h->at<float>(h->L.ctrl_add);
     if (pm1 >= 0) A.PM1 = ring_grid(h, h->pm, pm1);
     if (ub1 >= 0) A.UB1 = ring_grid(h, h->ub, ub1);
     if (pm0 >= 0) A.PM0 = ring_grid(h, h->pm, pm0);
@@ -772,41 +775,45 @@ struct Launcher {
     return e;
   }
 
-  // closed-loop controller at step t: sense state st and evaluate the MLP, giving row t of
-  // the actuation table (direct launches only: the persistent form is off with a controller)
+  // closed-loop controller at step t: evaluate the MLP on the state's sensor sums (of state st if
+  // given, else left by the G2P pass before), giving row t of the actuation table (direct
+  // launches only: the persistent form is off with a controller)
   cudaError_t ctrl_forward(int t, const float* st) {
     if (mode != kDirect) return cudaErrorNotSupported;
     const Dims& m = h->m;
     const Layout& L = h->L;
     const CtrlStep c = ctrl_step(h, t);
-    count += 2;
-    after_pass[sid()] = false;
+    count += st ? 2 : 1;
+    const bool early = after_pass[sid()] && !h->profile;
+    after_pass[sid()] = true;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_forward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off), st,
-                                 h->at<int>(L.group), h->at<double>(L.ctrl_part), h->at<float>(L.wact),
+                                 h->at<int>(L.group), h->at<float>(L.ctrl_part), h->at<float>(L.wact),
                                  h->at<double>(L.ctrl_u) + (size_t)t * m.S * m.ctrl_in,
                                  h->at<double>(L.ctrl_h) + (size_t)t * m.S * m.ctrl_H,
                                  h->at<double>(L.ctrl_y) + (size_t)t * m.S * m.G,
-                                 h->at<float>(L.act_tab) + (size_t)t * m.S * m.G, h->at<double>(L.ctrl_cnt), s);
+                                 h->at<float>(L.act_tab) + (size_t)t * m.S * m.G, h->at<double>(L.ctrl_cnt), early, s);
     });
   }
 
   // reverse of the controller at step t, after the P2G adjoint of step t left the
-  // per-tile actuation adjoints in wbar_tile and the adjoint of state t in adj
-  cudaError_t ctrl_backward(int t) {
+  // per-tile actuation adjoints in wbar_tile and the adjoint of state t in adj; apply: add the
+  // sensors' adjoints to it here (else the G2P adjoint that reads it does)
+  cudaError_t ctrl_backward(int t, bool apply) {
     if (mode != kDirect) return cudaErrorNotSupported;
     const Dims& m = h->m;
     const Layout& L = h->L;
     const CtrlStep c = ctrl_step(h, t);
-    count += 2;
-    after_pass[sid()] = false;
+    count += apply ? 2 : 1;
+    const bool early = after_pass[sid()] && !h->profile;
+    after_pass[sid()] = !apply;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_backward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off),
                                   h->at<int>(L.group), h->at<float>(L.wbar_tile), h->at<float>(L.wact),
                                   h->at<double>(L.ctrl_u) + (size_t)t * m.S * m.ctrl_in,
                                   h->at<double>(L.ctrl_h) + (size_t)t * m.S * m.ctrl_H,
                                   h->at<double>(L.ctrl_y) + (size_t)t * m.S * m.G, h->at<double>(L.ctrl_cnt),
-                                  h->at<double>(L.ctrl_thbar), h->at<float>(L.ctrl_add), h->at<float>(L.adj), s);
+                                  h->at<double>(L.ctrl_thbar), h->at<float>(L.ctrl_add), apply ? h->at<float>(L.adj) : nullptr, early, s);
     });
   }
 
@@ -1071,9 +1078,9 @@ int issue_forward_ctrl(mpm_handle* h, Launcher& Lc, int T) {
   LK(Lc.step(kP2GOnly, 0, src, nullptr, -1, &g, sL == 0 ? h->rslot(sL / K, 0) : nullptr));
   for (int t = 1; t < T; ++t) {
     float* dst = forward_stores_ckpt(h, T, t) ? h->ckpt(t / K) : (t > sL) ? h->seg(sL / K, t - sL) : cur;
-    LK(Lc.step(kG2POnlyFull, t, src, dst, g, nullptr));
+    LK(Lc.step(kG2POnlyFull, t, src, dst, g, nullptr, nullptr, true));
     ring_release(h->pm, g);
-    LK(Lc.ctrl_forward(t, dst));
+    LK(Lc.ctrl_forward(t, nullptr));
     LK(Lc.step(kP2GOnly, t, dst, nullptr, -1, &g, t >= sL ? h->rslot(sL / K, t - sL) : nullptr));
     src = dst;
   }
@@ -1124,13 +1131,13 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
       LK(Lc.adjoint(kAdjP2G, s, st_s1, st_s1, nullptr, pm_s1, ub_s1, -1, nullptr, nullptr, R1));
       ring_release(h->pm, pm_s1);
       ring_release(h->ub, ub_s1);
-      LK(Lc.ctrl_backward(s + 1));
+      LK(Lc.ctrl_backward(s + 1, false));
     } else if (h->m.words == 2) {  // deterministic: bound of the first ubar scatter
       LK(Lc.adjoint(kAdjG2P, s, st_s1, st_s, nullptr, -1, -1, pm_s, nullptr, nullptr, nullptr,
                     nullptr, 1));
     }
     int ub_s = -1;
-    LK(Lc.adjoint(kAdjG2P, s, st_s1, st_s, nullptr, -1, -1, pm_s, &ub_s, nullptr));
+    LK(Lc.adjoint(kAdjG2P, s, st_s1, st_s, nullptr, -1, -1, pm_s, &ub_s, nullptr, nullptr, nullptr, 0, s < T - 1));
     pm_s1 = pm_s;
     ub_s1 = ub_s;
   }
@@ -1138,7 +1145,7 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
   LK(Lc.adjoint(kAdjP2G, -1, st0, st0, nullptr, pm_s1, ub_s1, -1, nullptr, nullptr));
   ring_release(h->pm, pm_s1);
   ring_release(h->ub, ub_s1);
-  LK(Lc.ctrl_backward(0));
+  LK(Lc.ctrl_backward(0, true));
   LK(Lc.finish());
   return MPM_OK;
 }

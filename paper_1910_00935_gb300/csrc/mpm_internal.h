@@ -111,19 +111,22 @@ cudaError_t launch_loss_seed(int dim, int kind, int64_t N, int n_scenes, const i
 
 // controller.cu (closed-loop controller): sensing + MLP of one forward step, writing the
 // step's inputs u, hidden h, pre-scale outputs y, actuation act[scene][G] and group sizes
-// cnt[scene][G+1]; part: n_tiles x (G+1) x 7 doubles
+// cnt[scene][G+1]; part: n_tiles x (G+1) x (2 dim + 1) floats, the tiles' sensor sums -- of state st
+// if given (sensed here), else left by that state's G2P pass (StepArgs::sense).  early: may start
+// while the pass before it on the stream drains
 cudaError_t launch_ctrl_forward(const CtrlStep& cs, int n_scenes, int n_tiles, int64_t N,
                                 const int4* tiles, const int* tile_off, const float* st,
-                                const int* group, double* part, const float* theta, double* u,
-                                double* h, double* y, float* act, double* cnt, cudaStream_t s);
+                                const int* group, float* part, const float* theta, double* u,
+                                double* h, double* y, float* act, double* cnt, bool early, cudaStream_t s);
 // reverse of one step: reads (and clears) the per-tile actuation adjoints abar_tile[tile][G],
-// accumulates dL/dtheta into thbar (FP64) and adds the sensor terms to the x and v rows of
-// the state adjoint adj; add: n_scenes x (G+1) x 2 dim floats of scratch
+// accumulates dL/dtheta into thbar (FP64) and writes the sensor terms of the x and v rows of
+// the state adjoint to add (n_scenes x (G+1) x 2 dim floats), added to adj if given, else by the
+// G2P adjoint that reads it (AdjArgs::sense_add)
 cudaError_t launch_ctrl_backward(const CtrlStep& cs, int n_scenes, int n_tiles, int64_t N,
                                  const int4* tiles, const int* tile_off, const int* group,
                                  float* abar_tile, const float* theta, const double* u,
                                  const double* h, const double* y, const double* cnt,
-                                 double* thbar, float* add, float* adj, cudaStream_t s);
+                                 double* thbar, float* add, float* adj, bool early, cudaStream_t s);
 cudaError_t launch_ctrl_grad_out(int64_t n, const double* thbar, float* gw, cudaStream_t s);
 
 }  // namespace mpm

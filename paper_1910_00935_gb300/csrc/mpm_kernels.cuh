@@ -73,6 +73,7 @@ struct StepArgs {
   unsigned* err;
   unsigned long long* box_stats;  // [2]: gather boxes staged, of which too large for the shared
                                   // box (read from the grid instead); null: not counted
+  float* sense;            // closed-loop controller: per-tile sensor sums [tile][slot][value] (or null)
   int early;               // launched as a programmatic dependent (host only)
 };
 
@@ -110,6 +111,7 @@ struct AdjArgs {
   int* box_m_reset;
   Clears clears;
   unsigned* err;
+  const float* sense_add;  // kAdjG2P: sensor adjoints [scene][slot][2D] added to xbar, vbar (or null)
   int early;  // launched as a programmatic dependent (host only)
 };
 
@@ -753,6 +755,55 @@ __device__ __forceinline__ void reset_box(int* box, int scene) {
 }
 
 // ---------------------------------------------------------------------------
+// closed-loop controller: a tile's sums of x, v and the particle count by group slot (slot 0:
+// particles in no group), out[slot][x_0.., v_0.., count], in a fixed order: each warp sums
+// its lanes of one slot at a time (butterfly), then the warps are added in order.  Every
+// thread calls it.  scratch: kWarps * slots * (2D + 1) floats.
+// ---------------------------------------------------------------------------
+template <int D>
+__device__ __forceinline__ void sense_tile(int G, bool xfix, const int* group, bool active, int64_t p, const float x[D],
+                                           const float v[D], float* scratch, float* out) {
+  constexpr int NV = 2 * D + 1;
+  const int lane = threadIdx.x & 31, ns = G + 1;
+  int slot = -1;
+  if (active) {
+    const int g = group[p];
+    slot = (g >= 0 && g < G) ? g + 1 : 0;
+  }
+  float q[2 * D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    q[a] = xfix ? (float)__float_as_int(x[a]) * (1.0f / kFixPos) : x[a];
+    q[D + a] = v[a];
+  }
+  float* w = scratch + (threadIdx.x >> 5) * ns * NV;
+  for (int l = lane; l < ns * NV; l += 32) w[l] = 0.0f;
+  __syncwarp();
+  unsigned left = __ballot_sync(0xffffffffu, active);
+  while (left) {  // usually one or two slots a warp
+    const int s = __shfl_sync(0xffffffffu, slot, __ffs(left) - 1);
+    const bool in = slot == s;
+    const unsigned mask = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+    for (int c = 0; c < 2 * D; ++c) {
+      float t = in ? q[c] : 0.0f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == c) w[s * NV + c] = t;
+    }
+    if (lane == 2 * D) w[s * NV + 2 * D] = (float)__popc(mask);
+    left &= ~mask;
+  }
+  __syncthreads();
+  for (int l = threadIdx.x; l < ns * NV; l += kTile) {
+    float t = scratch[l];
+#pragma unroll
+    for (int k = 1; k < kWarps; ++k) t += scratch[k * ns * NV + l];
+    out[l] = t;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // P2G of the CTA's particles: stress, affine matrix A = kappa tau + m C, scatter
 // (m, m v + A dpos) into the scene grid g, fold the touched box into box_scene.
 // Every thread calls it; wb has not been used since an earlier barrier.
@@ -976,6 +1027,9 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     }
   }
 
+  if (MODE == kG2POnlyFull && A.sense)
+    sense_tile<D>(P.n_groups, P.xfix, A.group, active, p, x, v, reinterpret_cast<float*>(rec),
+                  A.sense + (int64_t)tile_index * (P.n_groups + 1) * (2 * D + 1));
   if (MODE != kG2POnlyFull) {
     stage_wait<0>();
     if (NC && MODE == kP2GOnly) pass_ready();
@@ -1081,6 +1135,15 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     for (int a = 0; a < D; ++a) vb[a] = A.adj[(R::V + a) * N + p];
 #pragma unroll
     for (int i = 0; i < D * D; ++i) Cb[i / D][i % D] = A.adj[(R::C + i) * N + p];
+    if (A.sense_add) {
+      const int g = A.group[p];
+      const float* add = A.sense_add + ((int64_t)scene * (P.n_groups + 1) + ((g >= 0 && g < P.n_groups) ? g + 1 : 0)) * 2 * D;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        xb[a] += add[a];
+        vb[a] += add[D + a];
+      }
+    }
   } else {
     // ---- P2G adjoint of step s+1: gather (pbar, mbar) = grid_op.grad(ubar, (m, p)) ----
     float x[D], v[D], E[D][D];
