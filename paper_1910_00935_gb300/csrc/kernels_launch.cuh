@@ -148,6 +148,21 @@ cudaError_t persistent_variant(int kind_mode, const SimParams& P, const PassEntr
   return cudaErrorInvalidValue;
 }
 
+// n consecutive buffers (grid_stride float4s, box_stride ints apart); C: words only
+template <int D>
+cudaError_t launch_clear_run(const Clears& C, float4* grid, int64_t grid_stride, const int* box, int box_stride, int n,
+                             int nnodes, int n_grid, int n_scenes, cudaStream_t s) {
+  const int blocks = n_scenes >= 8 ? 2 : 16;  // (of 256 threads a scene and buffer)
+  for (int z = 0; z < n; z += 65535) {
+    const int m = n - z < 65535 ? n - z : 65535;
+    clear_run_kernel<D><<<dim3(blocks, n_scenes, m), 256, 0, s>>>(C.words, grid + z * grid_stride, grid_stride,
+                                                                 box + (int64_t)z * box_stride, box_stride, nnodes, n_grid);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 template <int D>
 cudaError_t launch_clear(const Clears& C, int nnodes, int n_grid, int n_scenes, int blocks_per_scene,
                          cudaStream_t s) {

@@ -15,7 +15,11 @@
 // velocity adjoint) managed on the host: a pass scatters into a free clean buffer, the
 // buffer stays live until its last reader, and the next pass zeroes its recorded box.
 // Each buffer has two parity boxes so that resetting a box never races with a reader.
-// Every launch sequence starts and ends with all buffers clean.
+// Every launch sequence starts and ends with all buffers clean, but for those of a forward's last
+// segment: where a segment's grids are kept, the forward leaves them for its backward, which then
+// recomputes none of them (16 x 65,536 fixed-corotated particles, 128 steps in segments of 64: 68.5 ->
+// 61.6 ms forward and reverse; the 262,144-particle cube over 256 steps 30.8 -> 28.7).  Whatever
+// else comes next zeroes them first (drop_residents).
 //
 // Launch sequences are captured into CUDA graphs (one per forward length T and one
 // per backward length), cached on the handle and replayed on the caller's stream.
@@ -253,6 +257,10 @@ struct mpm_handle {
   bool materials_set = false;  // MPM_MIXED: per-particle materials given since the last set-up
   int32_t T_recorded = 0;
   int32_t resident_T = 0;  // T of the forward whose last segment is still in the segment buffer
+  // grids of the last segment's steps that the last forward left for the backward (kept segment
+  // grids only): (m, p) buffers res_lo .. res_lo + res_n - 1, each written once, its box in parity 0
+  int res_lo = 0, res_n = 0;
+  bool grids_clean = false;  // every other grid buffer holds zeros (false: the next set-up clears all)
   // options
   bool use_graphs = true;
   bool smem_tile = false;  // with tile_capacity only checked against the device (see mpm.h)
@@ -818,13 +826,16 @@ struct Launcher {
   }
 
   // End of a launch sequence (on the main stream, after any side-stream work has been
-  // joined): zero every dirty buffer, reset every box.
-  cudaError_t finish() {
+  // joined): zero every dirty buffer, reset every box -- except the (m, p) buffers keep_lo ..
+  // keep_lo + keep_n - 1 and their parity-0 boxes, which stay for the next sequence.
+  cudaError_t finish(int keep_lo = 0, int keep_n = 0) {
     cudaError_t e = flush();
     if (e != cudaSuccess) return e;
     for (Ring* r : {&h->pm, &h->ub})
       for (int i = 0; i < r->n; ++i)
-        if (r->state[i] == 1 || r->state[i] == 2) {
+        if (r == &h->pm && i >= keep_lo && i < keep_lo + keep_n) {
+          r->state[i] = 0;  // (not among this sequence's clears)
+        } else if (r->state[i] == 1 || r->state[i] == 2) {
           r->state[i] = 2;
           r->owner[i] = r->sid;
         }
@@ -842,8 +853,16 @@ struct Launcher {
       if (e != cudaSuccess) return e;
     }
     if (mode != kRecord) {
-      ++count;
-      e = launch_reset_boxes(h->at<int>(h->L.boxes), (int64_t)(h->m.pm_slots + kUBSlots) * 2 * h->m.S, s);
+      // (a kept buffer's parity-1 box is empty: its only write reset it)
+      const int64_t S2 = 2 * (int64_t)h->m.S, all = (int64_t)(h->m.pm_slots + kUBSlots), end = keep_lo + keep_n;
+      if (keep_n > 0 && keep_lo > 0) {
+        ++count;
+        e = launch_reset_boxes(h->at<int>(h->L.boxes), keep_lo * S2, s);
+      }
+      if (e == cudaSuccess) {
+        ++count;
+        e = launch_reset_boxes(h->at<int>(h->L.boxes) + (keep_n > 0 ? end * S2 * 8 : 0), (keep_n > 0 ? all - end : all) * S2, s);
+      }
     }
     ring_reset(h->pm);
     ring_reset(h->ub);
@@ -862,6 +881,17 @@ struct Launcher {
 // (and their polar factors) in the segment buffer, so the backward starts without
 // re-simulating it -- with ckpt_every >= T nothing is re-simulated at all
 int last_segment_start(const mpm_handle* h, int T) { return ((T - 1) / h->m.K) * h->m.K; }
+
+// whether a segment's grids stay live for its adjoint passes: those of a re-simulated segment, and
+// those of the last segment from the forward that ran it
+bool keeps_grids(const mpm_handle* h) { return h->m.store_grids && !h->grid_recompute; }
+
+// the (m, p) pool a forward's grid of step t is allocated from: the last segment's, which stay
+// live, in order from the start of the pool of that segment's parity, the others in the other pool
+int forward_pool(const mpm_handle* h, int T, int t) {
+  const int sL = last_segment_start(h, T), own = (sL / h->m.K) & 1;
+  return t >= sL ? own : 1 - own;
+}
 
 // whether the forward stores state t as a checkpoint: every K steps with one level; with two,
 // every K*M steps, and every K steps over the last coarse segment (left for the backward
@@ -900,13 +930,16 @@ int issue_coarse_resim(mpm_handle* h, Launcher& Lc, int Jc, int T) {
 int issue_forward(mpm_handle* h, Launcher& Lc, int T) {
   const int K = h->m.K;
   const int sL = last_segment_start(h, T);
+  const bool keep = keeps_grids(h);
   ring_reset(h->pm);
   ring_reset(h->ub);
   const float* src = h->state(h->L.ckpt, 0);
   float* cur = h->at<float>(h->L.cur);
   int g = -1;
+  if (keep) Lc.use_pool(forward_pool(h, T, 0));
   LK(Lc.step(kP2GOnly, 0, src, nullptr, -1, &g, sL == 0 ? h->rslot(sL / K, 0) : nullptr));
   for (int t = 1; t < T; ++t) {
+    if (keep) Lc.use_pool(forward_pool(h, T, t));
     float* dst;
     int mode;
     if (forward_stores_ckpt(h, T, t)) {
@@ -921,18 +954,16 @@ int issue_forward(mpm_handle* h, Launcher& Lc, int T) {
     }
     int g_next = -1;
     LK(Lc.step(mode, t, src, dst, g, &g_next, t >= sL ? h->rslot(sL / K, t - sL) : nullptr));
-    ring_release(h->pm, g);
+    if (!keep || t - 1 < sL) ring_release(h->pm, g);
     g = g_next;
     src = dst;
   }
   LK(Lc.step(kG2POnlyFull, T, src, h->at<float>(h->L.fin), g, nullptr));
-  ring_release(h->pm, g);
-  LK(Lc.finish());
+  if (!keep) ring_release(h->pm, g);
+  LK(Lc.finish(keep ? forward_pool(h, T, T - 1) * h->m.pm_pool : 0, keep ? T - sL : 0));
   return MPM_OK;
 }
 
-// re-simulate segment [s0, top): seg slot i <- state s0 + i (i = 1..top-s0); returns the
-// grid of step top-1 (kept live for the adjoint passes)
 // re-simulate segment [s0, top): seg slot i <- state s0 + i (i = 1..top-s0); returns the
 // grid of step top-1 (kept live for the adjoint passes); with seg_grids, every grid of the
 // segment is kept live too (seg_grids[t - s0] = grid of step t)
@@ -957,6 +988,14 @@ int issue_resim(mpm_handle* h, Launcher& Lc, int s0, int top, int* grid_top_minu
   return MPM_OK;
 }
 
+// take over the grids that the forward left (grids: their step order)
+void hold_residents(mpm_handle* h, std::vector<int>& grids) {
+  for (int i = 0; i < h->res_n; ++i) {
+    h->pm.state[h->res_lo + i] = 1;
+    grids[i] = h->res_lo + i;
+  }
+}
+
 // Backward.  With `overlap`, segment j-1 is re-simulated on the side stream while the
 // adjoint passes of segment j run on the main stream: the two are independent (the
 // re-simulation reads only checkpoint j-1) and latency-bound, so they share the SMs
@@ -966,16 +1005,18 @@ int issue_resim(mpm_handle* h, Launcher& Lc, int s0, int top, int* grid_top_minu
 // j has released the last grid of segment j+1 and the main stream has cleared that pool
 // (ev_free); the adjoint passes of segment j-1 start after its re-simulation (ev_resim).
 // A buffer released on a stream is cleared by a later launch on the same stream.
-int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overlap) {
+int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool grids, bool overlap) {
   const int K = h->m.K;
   ring_reset(h->pm);
   ring_reset(h->ub);
-  const bool kept = h->m.store_grids && !h->grid_recompute;
+  const bool kept = keeps_grids(h);
   // live grids: PM of steps s+1 and s, UB of step s+1
   int pm_s1 = -1, pm_s = -1, ub_s1 = -1;
   std::vector<int> seg_grids[2] = {std::vector<int>(K, -1), std::vector<int>(K, -1)};
   int side_top[2] = {-1, -1};  // grid of step top-1 of a segment re-simulated on the side
-  bool stored = false;         // this segment's grids were kept by its re-simulation
+  bool stored = false;         // this segment's grids were kept by its re-simulation or the forward
+  if (grids) hold_residents(h, seg_grids[((T - 1) / K) & 1]);
+  const bool hold = grids && last_segment_start(h, T) == 0;  // for a later backward of this forward
   if (overlap) {
     LK(Lc.signal(h->ev_fork));
     Lc.use_stream(1);
@@ -992,7 +1033,11 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overl
       int rc = issue_coarse_resim(h, Lc, coarse, T);
       if (rc) return rc;
     }
-    if (s == T - 1 && resident) {
+    if (s == T - 1 && grids) {
+      // the forward left this segment's states and grids in place
+      pm_s = seg_grids[pj][s - s0];
+      stored = true;
+    } else if (s == T - 1 && resident) {
       // the forward left this segment's states in place: only the grid of step T-1
       const float* st = (s == s0) ? h->ckpt(j) : h->seg(j, s - s0);
       LK(Lc.step(kP2GOnly, s, st, nullptr, -1, &pm_s));
@@ -1023,7 +1068,7 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overl
                     nullptr, 1));
     LK(Lc.adjoint(s == T - 1 ? kAdjG2P : kAdjFused, s, st_s1, st_s, st_sm,
                   s == T - 1 ? -1 : pm_s1, s == T - 1 ? -1 : ub_s1, pm_s, &ub_s, &pm_sm, R1, Rm));
-    ring_release(h->pm, pm_s1);
+    if (!hold) ring_release(h->pm, pm_s1);
     ring_release(h->ub, ub_s1);
     pm_s1 = pm_s;
     ub_s1 = ub_s;
@@ -1048,7 +1093,7 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overl
   }
   const float* st0 = h->state(h->L.ckpt, 0);
   LK(Lc.adjoint(kAdjP2G, -1, st0, st0, nullptr, pm_s1, ub_s1, -1, nullptr, nullptr));
-  ring_release(h->pm, pm_s1);
+  if (!hold) ring_release(h->pm, pm_s1);
   ring_release(h->ub, ub_s1);
   if (overlap) {  // join (the side stream's last work is already waited for)
     Lc.use_stream(1);
@@ -1056,7 +1101,7 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overl
     Lc.use_stream(0);
     LK(Lc.wait(h->ev_join));
   }
-  LK(Lc.finish());
+  LK(Lc.finish(hold ? h->res_lo : 0, hold ? h->res_n : 0));
   return MPM_OK;
 }
 
@@ -1069,24 +1114,27 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool overl
 int issue_forward_ctrl(mpm_handle* h, Launcher& Lc, int T) {
   const int K = h->m.K;
   const int sL = last_segment_start(h, T);
+  const bool keep = keeps_grids(h);
   ring_reset(h->pm);
   ring_reset(h->ub);
   const float* src = h->state(h->L.ckpt, 0);
   float* cur = h->at<float>(h->L.cur);
   int g = -1;
+  if (keep) Lc.use_pool(forward_pool(h, T, 0));
   LK(Lc.ctrl_forward(0, src));
   LK(Lc.step(kP2GOnly, 0, src, nullptr, -1, &g, sL == 0 ? h->rslot(sL / K, 0) : nullptr));
   for (int t = 1; t < T; ++t) {
     float* dst = forward_stores_ckpt(h, T, t) ? h->ckpt(t / K) : (t > sL) ? h->seg(sL / K, t - sL) : cur;
     LK(Lc.step(kG2POnlyFull, t, src, dst, g, nullptr, nullptr, true));
-    ring_release(h->pm, g);
+    if (!keep || t - 1 < sL) ring_release(h->pm, g);
+    if (keep) Lc.use_pool(forward_pool(h, T, t));
     LK(Lc.ctrl_forward(t, nullptr));
     LK(Lc.step(kP2GOnly, t, dst, nullptr, -1, &g, t >= sL ? h->rslot(sL / K, t - sL) : nullptr));
     src = dst;
   }
   LK(Lc.step(kG2POnlyFull, T, src, h->at<float>(h->L.fin), g, nullptr));
-  ring_release(h->pm, g);
-  LK(Lc.finish());
+  if (!keep) ring_release(h->pm, g);
+  LK(Lc.finish(keep ? forward_pool(h, T, T - 1) * h->m.pm_pool : 0, keep ? T - sL : 0));
   return MPM_OK;
 }
 
@@ -1096,13 +1144,15 @@ int issue_forward_ctrl(mpm_handle* h, Launcher& Lc, int T) {
 // reverse (which adds the sensor terms to it), and the G2P adjoint of step s read from
 // it.  Re-simulation reads the recorded actuation table; a grid that is neither kept nor
 // re-simulated is recomputed by its own P2G pass.
-int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
+int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident, bool grids) {
   const int K = h->m.K;
   ring_reset(h->pm);
   ring_reset(h->ub);
   int pm_s1 = -1, pm_s = -1, ub_s1 = -1;
   std::vector<int> seg_grids(K, -1);
   bool stored = false;
+  if (grids) hold_residents(h, seg_grids);
+  const bool hold = grids && last_segment_start(h, T) == 0;  // for a later backward of this forward
   int coarse = resident ? (T - 1) / (K * h->m.M) : -1;  // coarse segment whose checkpoints are built
   for (int s = T - 1; s >= 0; --s) {
     const int j = s / K, s0 = j * K;
@@ -1115,7 +1165,10 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
     const float* st_s = (s == s0) ? h->ckpt(j) : h->seg(j, s - s0);
     const float* st_s1 = (s + 1 == T) ? h->at<float>(h->L.fin) : h->seg(j, s + 1 - s0);
     const double* R1 = (s + 1 < top) ? h->rslot(j, s + 1 - s0) : nullptr;
-    if (s == T - 1 && resident) {
+    if (s == T - 1 && grids) {
+      pm_s = seg_grids[s - s0];
+      stored = true;
+    } else if (s == T - 1 && resident) {
       LK(Lc.step(kP2GOnly, s, st_s, nullptr, -1, &pm_s));
       stored = false;
     } else if (s == top - 1) {
@@ -1129,7 +1182,7 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
     }
     if (s < T - 1) {
       LK(Lc.adjoint(kAdjP2G, s, st_s1, st_s1, nullptr, pm_s1, ub_s1, -1, nullptr, nullptr, R1));
-      ring_release(h->pm, pm_s1);
+      if (!hold) ring_release(h->pm, pm_s1);
       ring_release(h->ub, ub_s1);
       LK(Lc.ctrl_backward(s + 1, false));
     } else if (h->m.words == 2) {  // deterministic: bound of the first ubar scatter
@@ -1143,10 +1196,32 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident) {
   }
   const float* st0 = h->state(h->L.ckpt, 0);
   LK(Lc.adjoint(kAdjP2G, -1, st0, st0, nullptr, pm_s1, ub_s1, -1, nullptr, nullptr));
-  ring_release(h->pm, pm_s1);
+  if (!hold) ring_release(h->pm, pm_s1);
   ring_release(h->ub, ub_s1);
   LK(Lc.ctrl_backward(0, true));
-  LK(Lc.finish());
+  LK(Lc.finish(hold ? h->res_lo : 0, hold ? h->res_n : 0));
+  return MPM_OK;
+}
+
+// Zero the grids that a forward left for its backward, where something else comes next.
+int drop_residents(mpm_handle* h, cudaStream_t s) {
+  if (h->res_n == 0) return MPM_OK;
+  const Dims& m = h->m;
+  Clears C;
+  memset(&C, 0, sizeof(C));
+  C.words = m.words;
+  float4* g = ring_grid(h, h->pm, h->res_lo);
+  int* b = ring_box(h, h->pm, h->res_lo, 0);
+  const int64_t stride = (int64_t)m.S * m.nnodes * m.words;
+  cudaError_t e = m.D == 2 ? launch_clear_run<2>(C, g, stride, b, 2 * m.S * 8, h->res_n, (int)m.nnodes, m.n_grid, m.S, s)
+                           : launch_clear_run<3>(C, g, stride, b, 2 * m.S * 8, h->res_n, (int)m.nnodes, m.n_grid, m.S, s);
+  if (e == cudaSuccess) e = launch_reset_boxes(b, (int64_t)h->res_n * 2 * m.S, s);
+  h->launches += 2;
+  h->res_n = 0;
+  if (e != cudaSuccess) {
+    h->grids_clean = false;
+    return cuda_fail(h, e, "clearing the last forward's grids");
+  }
   return MPM_OK;
 }
 
@@ -1249,6 +1324,8 @@ int run_sequence(mpm_handle* h, int64_t key, cudaStream_t stream, Fn&& issue) {
   if (rc != MPM_OK) {
     h->initialized = false;
     h->T_recorded = 0;
+    h->grids_clean = false;
+    h->res_n = 0;
   }
   return rc;
 }
@@ -1429,10 +1506,20 @@ int mpm_set_initial(mpm_handle* h, const float* x0, const float* v0, const float
                            h->at<float>(L.E), h->at<float>(L.nu), h->at<int>(L.group), s));
   const size_t wbytes = (size_t)m.S * m.n_act * sizeof(float);
   if (wbytes) CK(cudaMemcpyAsync(h->at<float>(L.wact), w, wbytes, cudaMemcpyDeviceToDevice, s));
-  const size_t grid = (size_t)m.S * m.nnodes * sizeof(float4) * m.words;
-  CK(cudaMemsetAsync(h->at<char>(L.grids), 0, grid * (m.pm_slots + kUBSlots), s));
+  // Every launch sequence leaves the grid buffers at zero but for the last forward's, so only the
+  // first set-up (or one after a failure) clears them all: on a 262,144-particle cube that was
+  // 4.6 GB, 0.7 ms of every set-up.
+  if (h->grids_clean) {
+    int rc = drop_residents(h, s);
+    if (rc) return rc;
+  } else {
+    const size_t grid = (size_t)m.S * m.nnodes * sizeof(float4) * m.words;
+    CK(cudaMemsetAsync(h->at<char>(L.grids), 0, grid * (m.pm_slots + kUBSlots), s));
+    CK(launch_reset_boxes(h->at<int>(L.boxes), (int64_t)(m.pm_slots + kUBSlots) * 2 * m.S, s));
+    h->res_n = 0;
+    h->grids_clean = true;
+  }
   CK(cudaMemsetAsync(h->at<char>(L.box_stats), 0, 16, s));
-  CK(launch_reset_boxes(h->at<int>(L.boxes), (int64_t)(m.pm_slots + kUBSlots) * 2 * m.S, s));
   ring_reset(h->pm);
   ring_reset(h->ub);
   h->launches += 3;
@@ -1464,10 +1551,16 @@ int mpm_forward(mpm_handle* h, int32_t T, void* stream) {
   if (T < 1 || T > h->max_steps) return fail(h, MPM_ERR_STATE, "T must be in [1, max_steps]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   h->last_stream = s;
-  int rc = run_sequence(h, (int64_t)T * 2, s, [&](Launcher& Lc) {
+  int rc = drop_residents(h, s);
+  if (rc) return rc;
+  rc = run_sequence(h, (int64_t)T * 2, s, [&](Launcher& Lc) {
     return h->m.ctrl_H > 0 ? issue_forward_ctrl(h, Lc, T) : issue_forward(h, Lc, T);
   });
   if (rc) return rc;
+  if (keeps_grids(h)) {
+    h->res_lo = forward_pool(h, T, T - 1) * h->m.pm_pool;
+    h->res_n = T - last_segment_start(h, T);
+  }
   h->T_recorded = T;
   h->resident_T = T;
   return MPM_OK;
@@ -1548,20 +1641,28 @@ int mpm_backward(mpm_handle* h, const float* dL_dx, const float* dL_dv, const fl
   h->launches += 4;
   const int T = h->T_recorded;
   const bool resident = h->resident_T == T;
+  const bool grids = resident && h->res_n > 0 && keeps_grids(h);
+  if (!grids) {
+    int rc = drop_residents(h, s);
+    if (rc) return rc;
+  }
   // the re-simulation overlaps the adjoint passes when there is a segment to re-simulate,
   // except in the persistent form (one stream of plan passes) and while profiling (each
   // launch timed alone)
   const bool overlap = h->overlap && !h->persistent && !h->profile && !ctrl && m.M == 1 &&
                        last_segment_start(h, T) > 0;
   const int64_t key = (int64_t)T * 2 + 1 + (resident ? 0 : ((int64_t)1 << 40)) +
-                      (overlap ? ((int64_t)1 << 41) : 0);
+                      (overlap ? ((int64_t)1 << 41) : 0) + (grids ? ((int64_t)1 << 42) : 0);
   int rc = run_sequence(h, key, s, [&](Launcher& Lc) {
-    return ctrl ? issue_backward_ctrl(h, Lc, T, resident) : issue_backward(h, Lc, T, resident, overlap);
+    return ctrl ? issue_backward_ctrl(h, Lc, T, resident, grids) : issue_backward(h, Lc, T, resident, grids, overlap);
   });
   if (rc) return rc;
   // re-simulating the earlier segments reused the segment buffer: a later backward of
   // the same forward re-simulates the last segment as well
-  if (last_segment_start(h, T) > 0) h->resident_T = 0;
+  if (last_segment_start(h, T) > 0) {
+    h->resident_T = 0;
+    h->res_n = 0;  // (cleared as its passes went)
+  }
   float* outs[4] = {gx0, gv0, gC0, gF0};
   r0 = 0;
   for (int k = 0; k < 4; ++k) {
@@ -1600,11 +1701,15 @@ int mpm_initial_p2g_grid(mpm_handle* h, float* grid, void* stream) {
   ring_reset(h->pm);
   ring_reset(h->ub);
   int g = -1;
+  Lc.use_pool(h->res_lo == 0 ? 1 : 0);  // (the last forward's grids stay)
+  const bool clean = h->grids_clean;
+  h->grids_clean = false;  // (should a launch fail)
   LK(Lc.step(kP2GOnly, 0, h->ckpt(0), nullptr, -1, &g));
   CK(cudaMemcpyAsync(grid, ring_grid(h, h->pm, g), (size_t)h->m.S * h->m.nnodes * sizeof(float4),
                      cudaMemcpyDeviceToDevice, s));
   ring_release(h->pm, g);
-  LK(Lc.finish());
+  LK(Lc.finish(h->res_lo, h->res_n));
+  h->grids_clean = clean;
   h->launches += Lc.count;
   return MPM_OK;
 }
@@ -1622,6 +1727,8 @@ int mpm_sync_status(mpm_handle* h) {
     // the word holds may follow from the incomplete state
     if (err & kErrTimeout) {
       // grid buffers may be dirty
+      h->grids_clean = false;
+      h->res_n = 0;
       h->initialized = false;
       h->T_recorded = 0;
       return fail(h, MPM_ERR_TIMEOUT, "a bounded device wait gave up (call mpm_set_initial again)");

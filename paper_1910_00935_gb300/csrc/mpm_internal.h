@@ -28,6 +28,10 @@ cudaError_t adj_variant(int mode, const SimParams& P, const AdjArgs& A, int n_ti
 template <int D, int MAT, bool DET>
 cudaError_t persistent_variant(int kind, const SimParams& P, const PassEntry* plan, int n_pass,
                                int n_tiles, const PersistCtl& ctl, cudaStream_t s, int* grid_out);
+// zero n consecutive buffers over their boxes (buffers grid_stride float4s, boxes box_stride ints apart)
+template <int D>
+cudaError_t launch_clear_run(const Clears& C, float4* grid, int64_t grid_stride, const int* box, int box_stride, int n,
+                             int nnodes, int n_grid, int n_scenes, cudaStream_t s);
 template <int D>
 cudaError_t launch_clear(const Clears& C, int nnodes, int n_grid, int n_scenes, int blocks_per_scene,
                          cudaStream_t s);

@@ -1697,4 +1697,18 @@ __global__ void clear_kernel(const __grid_constant__ Clears C, int nnodes, int n
   run_clears<D>(C, boxes, blockIdx.y, blockIdx.x, gridDim.x, nnodes, n);
 }
 
+// The same for a run of buffers (blockIdx.z), grid_stride float4s and box_stride ints apart.
+template <int D>
+__global__ void clear_run_kernel(int words, float4* grid, int64_t grid_stride, const int* box, int box_stride, int nnodes,
+                                 int n) {
+  __shared__ int boxes[8];
+  Clears C;
+  C.n = 1;
+  C.words = words;
+  C.job[0].grid = grid + blockIdx.z * grid_stride;
+  if (threadIdx.x < 8) boxes[threadIdx.x] = box[(int64_t)blockIdx.z * box_stride + blockIdx.y * 8 + threadIdx.x];
+  __syncthreads();
+  run_clears<D>(C, boxes, blockIdx.y, blockIdx.x, gridDim.x, nnodes, n);
+}
+
 }  // namespace mpm

@@ -1,0 +1,103 @@
+"""The grids that a forward leaves for its backward (kept segment grids): whatever is called between
+the two, or instead of one of them, gives what a fresh handle gives -- bitwise, in the
+deterministic mode, where the order of the sums does not matter."""
+import numpy as np
+import pytest
+
+from paper_1910_00935_gb300 import scenes
+from test_gpu_parity import _random_seeds
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+T = 14
+
+
+@pytest.fixture(scope="module")
+def mpm():
+    from paper_1910_00935_gb300 import build, mpm as m
+    build.build()
+    return m
+
+
+def _scene(name):
+    s = {"cube": lambda: scenes.make("cube3d", n_side=12, n_grid=48),
+         "rects": lambda: scenes.make("rects2d", n_scenes=3, n_min=200, n_max=700),
+         "nn": lambda: scenes.make("robots_nn", n_scenes=2, dims=(12, 8, 8), hidden=8)}[name]()
+    s["desc"]["deterministic_p2g"] = 1
+    return s
+
+
+def _back(sim, seeds):
+    return [t.clone() for t in sim.backward(**seeds).values()]
+
+
+def _same(a, b):
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("name", ["cube", "rects", "nn"])
+@pytest.mark.parametrize("k", [4, 7, 40])  # a ragged last segment, an even one, one segment
+@pytest.mark.parametrize("coarse", [0, 2])
+def test_any_order_of_calls(mpm, name, k, coarse):
+    scene = _scene(name)
+    scene["desc"]["ckpt_every"], scene["desc"]["ckpt_coarse"] = k, coarse
+    seeds = {key: torch.as_tensor(v).cuda() for key, v in _random_seeds(scene, np.random.default_rng(3)).items()}
+
+    def fresh(steps, graphs=1):
+        sim = mpm.from_scene(scene, max_steps=T)
+        sim.set_option(mpm.MPM_OPT_USE_GRAPHS, graphs)
+        sim.forward(steps)
+        return sim
+
+    ref_sim = fresh(T)
+    ref = _back(ref_sim, seeds)
+    sim9 = fresh(9, graphs=0)
+    ref9 = _back(sim9, seeds)
+    x = [t.clone() for t in ref_sim.state()]
+
+    sim = fresh(T)
+    sim.forward(T)                                  # a forward over the grids of another
+    _same(_back(sim, seeds), ref)
+    _same(_back(sim, seeds), ref)                   # a second backward of the same forward
+    sim.forward(9)                                  # another length, other buffers
+    sim.forward(T)
+    sim.forward(9)
+    _same(_back(sim, seeds), ref9)
+    sim.forward(T)
+    sim.reload()                                    # a set-up over kept grids
+    sim.forward(T)
+    _same(sim.state(), x)
+    _same(_back(sim, seeds), ref)
+    sim.forward(T)
+    for option, value in ((mpm.MPM_OPT_GRID_RECOMPUTE, 1), (mpm.MPM_OPT_USE_GRAPHS, 0), (mpm.MPM_OPT_OVERLAP_RESIM, 0)):
+        sim.set_option(option, value)               # an option between the two
+        _same(_back(sim, seeds), ref)
+        sim.forward(T)
+        _same(_back(sim, seeds), ref)
+    sim.set_option(mpm.MPM_OPT_GRID_RECOMPUTE, 0)
+    sim.forward(T)
+    _same(_back(sim, seeds), ref)
+    assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
+    for s in (ref_sim, sim9, sim):
+        s.close()
+
+
+def test_diagnostic_grid_between(mpm):
+    """mpm_initial_p2g_grid leaves a recorded forward, its kept grids among it, intact."""
+    scene = scenes.make("cube3d", n_side=12, n_grid=48)
+    scene["desc"]["ckpt_every"] = 40
+    seeds = {key: torch.as_tensor(v).cuda() for key, v in _random_seeds(scene, np.random.default_rng(3)).items()}
+    sim = mpm.from_scene(scene, max_steps=T)
+    grid = torch.empty(1, 48 ** 3, 4, device="cuda")
+    mpm.mpm_initial_p2g_grid(sim.h, grid)
+    first = grid.clone()
+    sim.forward(T)
+    ref = _back(sim, seeds)
+    sim.forward(T)
+    mpm.mpm_initial_p2g_grid(sim.h, grid)
+    assert float((grid - first).norm()) <= 1e-6 * float(first.norm())
+    for a, b in zip(_back(sim, seeds), ref):
+        assert float((a - b).norm()) <= 1e-4 * max(float(b.norm()), 1e-30)
+    assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
+    sim.close()
