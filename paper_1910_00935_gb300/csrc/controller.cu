@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kTile) ctrl_sense_kernel(int G, int64_t N, con
     x[a] = st[(int64_t)a * N + p];  // fixed-point position rows
     v[a] = st[(int64_t)(D + a) * N + p];
   }
-  sense_tile<D>(G, true, group, active, p, x, v, scratch, part + (int64_t)blockIdx.x * (G + 1) * (2 * D + 1));
+  sense_tile<D>(G, true, group[p], active, x, v, scratch, part + (int64_t)blockIdx.x * (G + 1) * (2 * D + 1));
 }
 
 // One CTA per scene: reduce the scene's tile sums in order, form the inputs, run the MLP

@@ -13,7 +13,7 @@ namespace mpm {
 namespace {
 // Raise a kernel's dynamic shared-memory limit when static + dynamic may pass the default
 // 48 KB: the passes' static shared memory (box slots, group sums, the persistent forms' pass
-// entry) stays below 5 KB, so any dynamic size above 32 KB sets it.
+// entry) stays below 4.5 KB, so any dynamic size above 32 KB sets it.
 template <typename K>
 cudaError_t allow_smem(K k, size_t smem) {
   if (smem <= 32 * 1024) return cudaSuccess;

@@ -64,7 +64,7 @@ struct Layout {
   size_t tiles, scene_off, scene_tiles, scene_tile_off;
   size_t mu, la, E, nu, group, matid, wact, wbar_tile, mubar, labar;
   size_t fin, cur, ckpt, fine, seg, adj;
-  size_t rcache;  // 2 x (K+1) x [9][N] polar factors of a segment (3D FCR; R_hi, R_lo as FP32 pairs), by parity
+  size_t rcache;  // 2 x (K+1) x [9][N] polar factors of a segment (3D FCR; see polar_to_cache), by parity
   size_t grids;  // pm_slots + kUBSlots dense grids
   size_t boxes;  // (pm_slots + kUBSlots) x 2 parities x [scene][8]
   size_t err, box_stats, com, com_part, ub_m0;
@@ -1331,13 +1331,13 @@ int run_sequence(mpm_handle* h, int64_t key, cudaStream_t stream, Fn&& issue) {
 }
 
 // Dynamic shared memory the particle passes need with the handle's capacities, plus the
-// passes' static shared memory (below 5 KB), against the device's per-CTA limit.
+// passes' static shared memory (below 4.5 KB), against the device's per-CTA limit.
 bool capacities_fit(const mpm_handle* h, std::string* why) {
   if (h->smem_optin <= 0) return true;
   const int cap = std::max(h->gather_capacity, h->smem_tile && !h->desc.deterministic_p2g ? h->tile_capacity : 0);
   const size_t need = (h->m.D == 2 ? std::max(step_smem_bytes<2>(cap), adj_smem_bytes<2>(cap))
                                    : std::max(step_smem_bytes<3>(cap), adj_smem_bytes<3>(cap))) +
-                      5 * 1024;
+                      4608;
   if (need <= (size_t)h->smem_optin) return true;
   char buf[160];
   snprintf(buf, sizeof(buf), "the shared node boxes need %zu B of shared memory per CTA, the device allows %d B",

@@ -370,7 +370,7 @@ __device__ __forceinline__ void plus_identity(const float E[D][D], float F[D][D]
 // ---------------------------------------------------------------------------
 template <int D>
 struct Polar {
-  float Rh[D][D], Rl[D][D];  // R = Rh + Rl to ~1e-14 (the per-segment cache stores both)
+  float Rh[D][D], Rl[D][D];  // R = Rh + Rl to ~1e-14
   float Rf[D][D];            // R rounded to FP32
   float Df[D][D];            // F - R formed from the exact parts, rounded once
 };
@@ -641,7 +641,7 @@ __host__ __device__ __forceinline__ bool polar_refine3(const float E[3][3], cons
 // as (c, s) / |(c, s)| in compensated FP32 (polar_refine2).
 // 3D: Newton's iteration in FP32 gives Q within FP32 resolution of R, refined without FP64
 // arithmetic (polar_refine3) to R = R_hi + R_lo and F - R; R in FP64 is formed from the pair
-// only where a pass needs it (the polar adjoint, the per-segment cache).  When the FP32 stage
+// only where a pass needs it (the FP64 variant's polar adjoint).  When the FP32 stage
 // fails (near-singular F) Newton's iteration runs in FP64 from F.
 // Returns false for det F <= 0 or non-finite input.
 template <int D>
@@ -790,9 +790,11 @@ __device__ __forceinline__ bool polar_factor(const float E[D][D], Polar<D>& p) {
   }
 }
 
-// The per-segment polar cache holds R_hi and R_lo as FP32 rows [2 D^2][N] (rows i*D + j,
-// then D^2 + i*D + j), in the footprint of [D^2][N] FP64 values; F - R is re-formed from them
-// exactly as the factorisation forms it.
+// The per-segment polar cache holds R rounded to FP32 and F - R as FP32 rows [2 D^2][N] (rows
+// i*D + j, then D^2 + i*D + j), all that the stress and the FP32 polar adjoint use: re-forming
+// F - R from R_hi and R_lo cost an adjoint pass ~300 of its 5,100 instructions a warp (4 of 276 us).  The FP64
+// variant's adjoint needs R itself: it keeps R_hi and R_lo and re-forms F - R exactly as the
+// factorisation forms it.
 template <int D>
 __device__ __forceinline__ void polar_from_cache(const double* Rc, int64_t N, int64_t p,
                                                  const float E[D][D], Polar<D>& pol) {
@@ -801,12 +803,17 @@ __device__ __forceinline__ void polar_from_cache(const double* Rc, int64_t N, in
   for (int i = 0; i < D; ++i)
 #pragma unroll
     for (int j = 0; j < D; ++j) {
-      const float rh = r[(int64_t)(i * D + j) * N + p];
-      const float rl = r[(int64_t)(D * D + i * D + j) * N + p];
-      pol.Rh[i][j] = rh;
-      pol.Rl[i][j] = rl;
-      pol.Rf[i][j] = rh + rl;
-      pol.Df[i][j] = f_minus_r(i == j ? 1.0f : 0.0f, E[i][j], rh, rl);
+      const float a = r[(int64_t)(i * D + j) * N + p];
+      const float b = r[(int64_t)(D * D + i * D + j) * N + p];
+#if MPM_POLAR_FP64
+      pol.Rh[i][j] = a;
+      pol.Rl[i][j] = b;
+      pol.Rf[i][j] = a + b;
+      pol.Df[i][j] = f_minus_r(i == j ? 1.0f : 0.0f, E[i][j], a, b);
+#else
+      pol.Rf[i][j] = a;
+      pol.Df[i][j] = b;
+#endif
     }
 }
 
@@ -817,8 +824,8 @@ __device__ __forceinline__ void polar_to_cache(double* Rc, int64_t N, int64_t p,
   for (int i = 0; i < D; ++i)
 #pragma unroll
     for (int j = 0; j < D; ++j) {
-      r[(int64_t)(i * D + j) * N + p] = pol.Rh[i][j];
-      r[(int64_t)(D * D + i * D + j) * N + p] = pol.Rl[i][j];
+      r[(int64_t)(i * D + j) * N + p] = MPM_POLAR_FP64 ? pol.Rh[i][j] : pol.Rf[i][j];
+      r[(int64_t)(D * D + i * D + j) * N + p] = MPM_POLAR_FP64 ? pol.Rl[i][j] : pol.Df[i][j];
     }
 }
 
@@ -978,8 +985,8 @@ __device__ __forceinline__ float column_of(const float row[D], int axis) {
 // tau += act (F e)(F e)^T, e = unit vector of `axis` (actuation fibre)
 // with F = I + E; every product is formed on E (or on F - R) so small strains keep
 // their relative precision.
-// Rc (fixed-corotated only, may be null): the cached polar factor of this particle (R_hi and
-// R_lo rows, particle p), used instead of recomputing it.
+// Rc (fixed-corotated only, may be null): the cached polar factor of this particle (rows of
+// polar_to_cache, particle p), used instead of recomputing it.
 template <int D, int MAT>
 __device__ __forceinline__ bool kirchhoff(const float E[D][D], float mu, float la, float act, int axis,
                                           float tau[D][D], StressCache<D>& sc,

@@ -66,7 +66,7 @@ struct StepArgs {
   const float* wact;       // [scene][group][basis]
   const float4* PMr;       // grid (m, p) of step t-1, read by G2P (null: P2G only)
   float4* PMw;             // grid of step t, accumulated by P2G (null: G2P only)
-  double* Rw;              // [9][N] polar factors (R_hi, R_lo pairs) of the P2G's states, written (or null)
+  double* Rw;              // [9][N] polar factors (polar_to_cache) of the P2G's states, written (or null)
   int* box_w;              // [scene][8] box of PMw for this use
   int* box_reset;          // [scene][8] the other parity box of PMw, reset here (or null)
   Clears clears;
@@ -157,6 +157,45 @@ __device__ __forceinline__ float4 ub_load(const float4* g, int64_t node, const S
 __device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pass_ready() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Packed FP32 pairs: one instruction for two independent operations, each rounded as on its own.
+// Used where a pass is short of issue slots: the 3D adjoint gathers (16 warps an SM; fused pass of
+// 16 x 65,536 fixed-corotated particles 276 -> 270 us, adjoint of the last step 138 -> 130).  In the
+// forward gather and the scatter they measured no gain.
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
+__device__ __forceinline__ float f2_lo(F2 p) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v));
+  return a;
+}
+__device__ __forceinline__ float f2_hi(F2 p) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v));
+  return b;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+
 struct NodePair {
   float4 ub, pm;
 };
@@ -188,14 +227,19 @@ constexpr int kWbarSlots = (kTile / 32) * kMaxGroups;
 // [r * kTile + threadIdx.x]; each thread copies and later reads only its own column.
 template <int D>
 struct Stage {
-  static constexpr int kStep = 2;                   // mu, la (read by the P2G stress)
+  static constexpr int kStep = 3;                   // mu, la, group (read by the P2G stress)
   static constexpr int kAdjB = D + D * D;           // x, F rows of state s (G2P-adjoint)
   static constexpr int kAdjC = 2 * D + 2 * D * D;   // full state s-1 (recomputed P2G)
-  static constexpr int kAdj = kAdjB + kAdjC + 2;    // + mu, la
+  static constexpr int kAdj = kAdjB + kAdjC + 3;    // + mu, la, group
 };
 __device__ __forceinline__ void stage_row(float* stage, int r, const float* src) {
   const unsigned dst = (unsigned)__cvta_generic_to_shared(stage + r * kTile + threadIdx.x);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+// a float2 of each particle into rows r and r + 1
+__device__ __forceinline__ void stage_pair(float* stage, int r, const float2* src) {
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(stage + r * kTile + 2 * threadIdx.x);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // wait until at most N of this thread's copy groups are still in flight (the passes use
@@ -203,6 +247,9 @@ __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_g
 template <int N>
 __device__ __forceinline__ void stage_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ float2 staged_pair(const float* stage, int r) {
+  return *reinterpret_cast<const float2*>(stage + r * kTile + 2 * threadIdx.x);
 }
 __device__ __forceinline__ float staged(const float* stage, int r) { return stage[r * kTile + threadIdx.x]; }
 
@@ -434,7 +481,7 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
 //   mass  W * mass_c          (when WITH_MASS)
 //   vec   W * (a + B dpos)
 // A particle's 3^D nodes are 3^(D-1) columns along the grid's last axis.  Each warp scatters
-// its own 32 particles: lane (slot, column) walks its slot's third (3D) or tenth (2D) of them
+// its own 32 particles: lane (slot, column) walks its slot's third (3D) or eighth (2D) of them
 // in order, sums their contributions to its column's three nodes in registers, and while the
 // stencil base moves along the last axis by a node or two only reduces the nodes that fall out
 // of the window into the grid; any other move reduces all three.  The particle order makes
@@ -642,12 +689,12 @@ __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n
   }
 }
 
-__device__ __forceinline__ float particle_act(const SimParams& P, const float* basis, const int* group,
-                                              const float* wact, int scene, int64_t p, int dim,
-                                              int& axis) {
+// actuation of a particle of group g (< 0 or >= n_groups: none) at a step with the given basis; axis:
+// the fibre's.  The group comes by an asynchronous copy issued before a pass waits for the one before it
+// (staged_group), so that its round trip is not on the chain of the stress.
+__device__ __forceinline__ float particle_act(const SimParams& P, const float* basis, int g,
+                                              const float* wact, int scene, int dim, int& axis) {
   axis = 0;
-  if (P.n_groups <= 0) return 0.0f;
-  int g = group[p];
   if (g < 0 || g >= P.n_groups) return 0.0f;
   axis = g % dim;
   const float* w = wact + ((int64_t)scene * P.n_groups + g) * P.n_basis;
@@ -656,6 +703,11 @@ __device__ __forceinline__ float particle_act(const SimParams& P, const float* b
   for (int k = 0; k < kMaxBasis; ++k)
     if (k < P.n_basis) a += w[k] * basis[k];
   return a;
+}
+
+// the particle's group from its staged row (-1: no groups)
+__device__ __forceinline__ int staged_group(const SimParams& P, const float* stage, int r) {
+  return P.n_groups > 0 ? __float_as_int(staged(stage, r)) : -1;
 }
 
 template <int D>
@@ -761,15 +813,11 @@ __device__ __forceinline__ void reset_box(int* box, int scene) {
 // thread calls it.  scratch: kWarps * slots * (2D + 1) floats.
 // ---------------------------------------------------------------------------
 template <int D>
-__device__ __forceinline__ void sense_tile(int G, bool xfix, const int* group, bool active, int64_t p, const float x[D],
-                                           const float v[D], float* scratch, float* out) {
+__device__ __forceinline__ void sense_tile(int G, bool xfix, int g, bool active, const float x[D], const float v[D],
+                                           float* scratch, float* out) {
   constexpr int NV = 2 * D + 1;
   const int lane = threadIdx.x & 31, ns = G + 1;
-  int slot = -1;
-  if (active) {
-    const int g = group[p];
-    slot = (g >= 0 && g < G) ? g + 1 : 0;
-  }
+  const int slot = !active ? -1 : (g >= 0 && g < G) ? g + 1 : 0;
   float q[2 * D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
@@ -810,10 +858,9 @@ __device__ __forceinline__ void sense_tile(int G, bool xfix, const int* group, b
 // ---------------------------------------------------------------------------
 template <int D, int MAT, bool DET>
 __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis, bool active, int scene,
-                                         int64_t p, const float x[D], const float v[D],
+                                         int64_t p, int grp, const float x[D], const float v[D],
                                          const float C[D][D], const float E[D][D], float mu_p,
-                                         float la_p, int mat_p, const int* group, const float* wact,
-                                         float4* g, int* box_scene, float4* rec, WarpBounds& wb,
+                                         float la_p, int mat_p, const float* wact, float4* g, int* box_scene, float4* rec, WarpBounds& wb,
                                          int seen, unsigned& err, const double* R_in, double* R_out, int64_t N) {
   Axes<D> s;
   bool ok = make_axes<D>(x, P, s) && active;
@@ -827,7 +874,7 @@ __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis,
   }
   if (ok) {
     int axis;
-    const float act = particle_act(P, basis, group, wact, scene, p, D, axis);
+    const float act = particle_act(P, basis, grp, wact, scene, D, axis);
     float tau[D][D];
     StressCache<D> sc;
     if (!kirchhoff<D, MAT>(E, mu_p, la_p, act, axis, tau, sc, R_in, N, p, mat_p)) {
@@ -883,6 +930,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     stage_row(stage, 0, A.mu + p);
     stage_row(stage, 1, A.la + p);
   }
+  if (P.n_groups > 0) stage_row(stage, 2, reinterpret_cast<const float*>(A.group) + p);
   const int nranks = A.scene_tiles[scene];
   if (NC) pass_wait();
   const int seen = MODE != kG2POnlyFull ? box_seen(A.box_w + scene * 8) : 0;
@@ -1028,14 +1076,13 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
   }
 
   if (MODE == kG2POnlyFull && A.sense)
-    sense_tile<D>(P.n_groups, P.xfix, A.group, active, p, x, v, reinterpret_cast<float*>(rec),
+    sense_tile<D>(P.n_groups, P.xfix, staged_group(P, stage, 2), active, x, v, reinterpret_cast<float*>(rec),
                   A.sense + (int64_t)tile_index * (P.n_groups + 1) * (2 * D + 1));
   if (MODE != kG2POnlyFull) {
     stage_wait<0>();
     if (NC && MODE == kP2GOnly) pass_ready();
-    p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, x, v, C, E, staged(stage, 0), staged(stage, 1),
-                          MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact, scene_grid(A.PMw, scene, P),
-                          A.box_w + scene * 8, rec, sh.scatter[0], seen, err, nullptr, A.Rw, N);
+    p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, staged_group(P, stage, 2), x, v, C, E, staged(stage, 0),
+                          staged(stage, 1), MAT == kMixed ? A.matid[p] : MAT, A.wact, scene_grid(A.PMw, scene, P), A.box_w + scene * 8, rec, sh.scatter[0], seen, err, nullptr, A.Rw, N);
     if (MODE == kP2GOnly) run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
   }
   if (err) atomicOr(A.err, err);
@@ -1082,6 +1129,8 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   const float c4 = 4.0f * P.inv_dx * P.inv_dx;
   unsigned err = 0;
   const int nranks = A.scene_tiles[scene];
+  float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
+  if (P.n_groups > 0) stage_row(stage, Stage<D>::kAdj - 1, reinterpret_cast<const float*>(A.group) + p);
   if (NC) pass_wait();
   const int seen_ub = MODE != kAdjP2G && A.box_ub ? box_seen(A.box_ub + scene * 8) : 0;
   const int seen_m = MODE != kAdjP2G && A.stm ? box_seen(A.box_m + scene * 8) : 0;
@@ -1093,7 +1142,6 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   }
   // stage what the G2P-adjoint (state s: x, F) and the recomputed P2G (state s-1, mu, la)
   // read, so that those loads are in flight during the P2G-adjoint
-  float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
   if (MODE != kAdjP2G) {
 #pragma unroll
     for (int a = 0; a < D; ++a) stage_row(stage, a, A.st0 + (int64_t)(R::X + a) * N + p);
@@ -1101,11 +1149,31 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     for (int i = 0; i < D * D; ++i) stage_row(stage, D + i, A.st0 + (int64_t)(R::F + i) * N + p);
   }
   stage_commit();
+  constexpr bool kCarried = D == 3 && MODE != kAdjG2P;
+  constexpr int kSums = D + 2 * D * D;
+  static_assert(D == 2 || kSums + 4 <= Stage<D>::kAdj - 1 - Stage<D>::kAdjB, "the carried rows fit");
   if (MODE != kAdjP2G && A.stm) {  // the recomputed P2G runs whenever state s-1 is given
 #pragma unroll
     for (int r = 0; r < R::Q; ++r) stage_row(stage, Stage<D>::kAdjB + r, A.stm + (int64_t)r * N + p);
     stage_row(stage, Stage<D>::kAdjB + R::Q, A.mu + p);
     stage_row(stage, Stage<D>::kAdjB + R::Q + 1, A.la + p);
+  }
+  // without it, its rows hold what the P2G-adjoint needs after its gather: the carried adjoint, C
+  // of state s+1, the material sums -- at four CTAs an SM each exposed round trip is ~3% of a
+  // tile's 33,000 cycles (with the group ahead of the chain and nothing waiting for the dL/dw
+  // slot, 16 x 65,536 fixed-corotated: fused pass 263 -> 250 us, last P2G-adjoint 215 -> 199)
+  const bool carried = kCarried && !A.stm;
+  if (carried) {
+    constexpr int b = Stage<D>::kAdjB;
+#pragma unroll
+    for (int a = 0; a < D; ++a) stage_row(stage, b + a, A.adj + (int64_t)(R::X + a) * N + p);
+#pragma unroll
+    for (int i = 0; i < D * D; ++i) {
+      stage_row(stage, b + D + i, A.adj + (int64_t)(R::F + i) * N + p);
+      stage_row(stage, b + D + D * D + i, A.st1 + (int64_t)(R::C + i) * N + p);
+    }
+    stage_pair(stage, b + kSums, A.mubar + p);
+    stage_pair(stage, b + kSums + 2, A.labar + p);
   }
   stage_commit();
 
@@ -1118,6 +1186,18 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   float xb[D], vb[D], Cb[D][D], Fb[D][D];
   float C1[D][D];
   auto load_carried = [&]() {
+    if (carried) {
+      stage_wait<0>();
+      constexpr int b = Stage<D>::kAdjB;
+#pragma unroll
+      for (int a = 0; a < D; ++a) xb[a] = staged(stage, b + a);
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) {
+        Fb[i / D][i % D] = staged(stage, b + D + i);
+        C1[i / D][i % D] = staged(stage, b + D + D * D + i);
+      }
+      return;
+    }
 #pragma unroll
     for (int a = 0; a < D; ++a) xb[a] = A.adj[(R::X + a) * N + p];
 #pragma unroll
@@ -1136,8 +1216,9 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
 #pragma unroll
     for (int i = 0; i < D * D; ++i) Cb[i / D][i % D] = A.adj[(R::C + i) * N + p];
     if (A.sense_add) {
-      const int g = A.group[p];
-      const float* add = A.sense_add + ((int64_t)scene * (P.n_groups + 1) + ((g >= 0 && g < P.n_groups) ? g + 1 : 0)) * 2 * D;
+      stage_wait<2>();
+      const int grp = staged_group(P, stage, Stage<D>::kAdj - 1);
+      const float* add = A.sense_add + ((int64_t)scene * (P.n_groups + 1) + ((grp >= 0 && grp < P.n_groups) ? grp + 1 : 0)) * 2 * D;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
         xb[a] += add[a];
@@ -1157,7 +1238,9 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     bool ok = make_axes<D>(x, P, s) && active;
     if (active && !ok) err |= kErrOOB;
     int axis;
-    const float act = particle_act(P, P.basis, A.group, A.wact, scene, p, D, axis);
+    stage_wait<2>();  // this thread's group and its share of the clear boxes, before the barrier below
+    const int grp = staged_group(P, stage, Stage<D>::kAdj - 1);
+    const float act = particle_act(P, P.basis, grp, A.wact, scene, D, axis);
     const float mu = A.mu[p], la = A.la[p];
     float tau[D][D];
     StressCache<D> sc;
@@ -1189,7 +1272,6 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     auto pbar = [&](const NodePair& g, bool wall) { return node_adjoint<D>(g.ub, g.pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
-    stage_wait<2>();  // this thread's share of the clear boxes, before the barrier below
     if (P.gather_capacity > 0) {
       gbx = box_extent<D>(ok, s.base, P.gather_capacity, sh.gather[0]);
       box_load<D, 2>(gbx, reinterpret_cast<float4*>(sm), P, raw, pbar);
@@ -1204,7 +1286,80 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       const float4 gc = load(1, 1, D == 3 ? 1 : 0);
       const float pc[3] = {gc.x, gc.y, gc.z};
       GatherAxes<D> ga(s);
-#pragma unroll(D == 3 ? 1 : 3)
+      if constexpr (D == 3) {
+        constexpr int Z = D - 1;
+        // pairs: components (0, 1) and (2, mass)
+        const F2 nc = f2(-gc.x, -gc.y), ncm = f2(-gc.z, -gc.w), z2 = f2(0.0f);
+        const F2 A0 = f2(Am[0][0], Am[1][0]), A1 = f2(Am[0][1], Am[1][1]), A2 = f2(Am[0][Z], Am[1][Z]);
+        F2 sw01 = z2, Ab0 = z2, Ab1 = z2, Ab2 = z2;
+        float swz = 0.0f, Ab0z = 0.0f, Ab1z = 0.0f, Ab2z = 0.0f;
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          float wi, dwi, dpi;
+          axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
+          const F2 qi = f2_fma(A0, f2(dpi), f2(mv[0], mv[1]));
+          const float qiz = mv[Z] + Am[Z][0] * dpi;
+          F2 t = z2, t1 = z2, t2 = z2;
+          float tz = 0.0f, t1z = 0.0f, t2z = 0.0f, e[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const F2 qij = f2_fma(A1, f2(s.dp[1][j]), qi);
+            const float qijz = qiz + Am[Z][1] * s.dp[1][j];
+            F2 r = z2, rb = z2;
+            float rz = 0.0f, rbz = 0.0f, e0 = 0.0f, e1 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const float4 g4 = load(i, j, k);
+              const F2 d = f2_add(f2(g4.x, g4.y), nc), dm = f2_add(f2(g4.z, g4.w), ncm);
+              const F2 q = f2_fma(A2, f2(s.dp[Z][k]), qij);
+              const F2 m = f2_fma(dm, f2(qijz + Am[Z][Z] * s.dp[Z][k], P.p_mass), f2_mul(d, q));
+              const float Wbar = f2_lo(m) + f2_hi(m), dz = f2_lo(dm);
+              r = f2_fma(f2(s.w[Z][k]), d, r);
+              rb = f2_fma(f2(ga.wp[Z][k]), d, rb);
+              rz += s.w[Z][k] * dz;
+              rbz += ga.wp[Z][k] * dz;
+              e0 += s.w[Z][k] * Wbar;
+              e1 += s.dw[Z][k] * Wbar;
+            }
+            const F2 w1 = f2(s.w[1][j]);
+            t = f2_fma(w1, r, t);
+            t1 = f2_fma(f2(ga.wp[1][j]), r, t1);
+            t2 = f2_fma(w1, rb, t2);
+            tz += s.w[1][j] * rz;
+            t1z += ga.wp[1][j] * rz;
+            t2z += s.w[1][j] * rbz;
+            e[0] += s.w[1][j] * e0;
+            e[1] += s.dw[1][j] * e0;
+            e[2] += s.w[1][j] * e1;
+          }
+          const float wpi = wi * dpi;
+          const F2 w0 = f2(wi);
+          sw01 = f2_fma(w0, t, sw01);
+          Ab0 = f2_fma(f2(wpi), t, Ab0);
+          Ab1 = f2_fma(w0, t1, Ab1);
+          Ab2 = f2_fma(w0, t2, Ab2);
+          swz += wi * tz;
+          Ab0z += wpi * tz;
+          Ab1z += wi * t1z;
+          Ab2z += wi * t2z;
+          xg[0] += dwi * e[0];
+          xg[1] += wi * e[1];
+          xg[Z] += wi * e[2];
+        }
+        sw[0] = f2_lo(sw01);
+        sw[1] = f2_hi(sw01);
+        sw[Z] = swz;
+        Ab[0][0] = f2_lo(Ab0);
+        Ab[1][0] = f2_hi(Ab0);
+        Ab[Z][0] = Ab0z;
+        Ab[0][1] = f2_lo(Ab1);
+        Ab[1][1] = f2_hi(Ab1);
+        Ab[Z][1] = Ab1z;
+        Ab[0][Z] = f2_lo(Ab2);
+        Ab[1][Z] = f2_hi(Ab2);
+        Ab[Z][Z] = Ab2z;
+      } else {
+#pragma unroll
       for (int i = 0; i < 3; ++i) {
         float wi, dwi, dpi, qi[D], t[D], tb[D][D], e[D];
         axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
@@ -1268,6 +1423,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
 #pragma unroll
         for (int b = 1; b < D; ++b) xg[b] += wi * e[b];
       }
+      }
 #pragma unroll
       for (int c = 0; c < D; ++c) vb[c] = pc[c] + sw[c];  // sum W = 1
     });
@@ -1300,7 +1456,8 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
     if (ok) abar = kirchhoff_adjoint<D, MAT>(E, A.mu[p], A.la[p], act, axis, sc, tb, Fb, mub, lab, mat_p);
     if (active) {
-      float2 ms = A.mubar[p], ls = A.labar[p];
+      float2 ms = carried ? staged_pair(stage, Stage<D>::kAdjB + kSums) : A.mubar[p];
+      float2 ls = carried ? staged_pair(stage, Stage<D>::kAdjB + kSums + 2) : A.labar[p];
       compensated_add(ms, mub);
       compensated_add(ls, lab);
       A.mubar[p] = ms;
@@ -1310,20 +1467,18 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       // dL/dw_gk += basis_k * sum of abar over this tile's particles of group g, reduced in
       // a fixed order (warp butterfly, then warps in order) into the tile's own slot, so
       // the result does not depend on scheduling; the tiles are summed in order at the end
-      int g = -1;
-      if (ok) {
-        g = A.group[p];
-        if (g < 0 || g >= P.n_groups) g = -1;
-      }
+      const int g = ok && grp < P.n_groups ? grp : -1;
       const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+      if (lane < kMaxGroups) s_wbar[warp * kMaxGroups + lane] = 0.0f;
+      __syncwarp();
+      unsigned left = __ballot_sync(0xffffffffu, g >= 0);
+      while (left) {  // the groups of the warp's particles: usually one
+        const int gg = __shfl_sync(0xffffffffu, g, __ffs(left) - 1);
+        float v = (g == gg) ? abar : 0.0f;
 #pragma unroll
-      for (int gg = 0; gg < kMaxGroups; ++gg) {
-        if (gg < P.n_groups) {
-          float v = (g == gg) ? abar : 0.0f;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-          if (lane == 0) s_wbar[warp * kMaxGroups + gg] = v;
-        }
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) s_wbar[warp * kMaxGroups + gg] = v;
+        left &= ~__ballot_sync(0xffffffffu, g == gg);
       }
       __syncthreads();
       const int GK = P.n_groups * P.n_basis;
@@ -1331,7 +1486,8 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
         const int gg = threadIdx.x / P.n_basis, k = threadIdx.x % P.n_basis;
         float sum = 0.0f;
         for (int w = 0; w < kTile / 32; ++w) sum += s_wbar[w * kMaxGroups + gg];
-        A.wbar_tile[(int64_t)tile_index * GK + threadIdx.x] += sum * P.basis[k];
+        // (the tile's own slot: a reduction only so that nothing waits for the value)
+        atomicAdd(A.wbar_tile + (int64_t)tile_index * GK + threadIdx.x, sum * P.basis[k]);
       }
     }
     if (MODE == kAdjP2G) {
@@ -1428,7 +1584,55 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       float xg[D], sw[D];
 #pragma unroll
       for (int a = 0; a < D; ++a) xg[a] = sw[a] = 0.0f;
-#pragma unroll(D == 3 ? 1 : 3)
+      if constexpr (D == 3) {
+        constexpr int Z = D - 1;
+        const F2 nc = f2(-uc[0], -uc[1]), z2 = f2(0.0f);
+        const F2 A0 = f2(c4 * Ct[0][0], c4 * Ct[1][0]), A1 = f2(c4 * Ct[0][1], c4 * Ct[1][1]), A2 = f2(c4 * Ct[0][Z], c4 * Ct[1][Z]);
+        F2 sw01 = z2;
+        float swz = 0.0f;
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          float wi, dwi, dpi;
+          axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
+          const F2 qi = f2_fma(A0, f2(dpi), f2(vt[0], vt[1]));
+          const float qiz = vt[Z] + c4 * Ct[Z][0] * dpi;
+          F2 t = z2;
+          float tz = 0.0f, e[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const F2 qij = f2_fma(A1, f2(s.dp[1][j]), qi);
+            const float qijz = qiz + c4 * Ct[Z][1] * s.dp[1][j];
+            F2 r = z2;
+            float rz = 0.0f, e0 = 0.0f, e1 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const float4 u4 = load(i, j, k);
+              const F2 d = f2_add(f2(u4.x, u4.y), nc);
+              const float dz = u4.z - uc[2];
+              const F2 m = f2_mul(d, f2_fma(A2, f2(s.dp[Z][k]), qij));
+              const float Wbar = dz * (qijz + c4 * Ct[Z][Z] * s.dp[Z][k]) + (f2_lo(m) + f2_hi(m));
+              r = f2_fma(f2(s.w[Z][k]), d, r);
+              rz += s.w[Z][k] * dz;
+              e0 += s.w[Z][k] * Wbar;
+              e1 += s.dw[Z][k] * Wbar;
+            }
+            t = f2_fma(f2(s.w[1][j]), r, t);
+            tz += s.w[1][j] * rz;
+            e[0] += s.w[1][j] * e0;
+            e[1] += s.dw[1][j] * e0;
+            e[2] += s.w[1][j] * e1;
+          }
+          sw01 = f2_fma(f2(wi), t, sw01);
+          swz += wi * tz;
+          xg[0] += dwi * e[0];
+          xg[1] += wi * e[1];
+          xg[Z] += wi * e[2];
+        }
+        sw[0] = f2_lo(sw01);
+        sw[1] = f2_hi(sw01);
+        sw[Z] = swz;
+      } else {
+#pragma unroll
       for (int i = 0; i < 3; ++i) {
         float wi, dwi, dpi, qi[D], t[D], e[D];
         axis_at(i, s.f[0], P.dx, wi, dwi, dpi);
@@ -1474,6 +1678,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
         xg[0] += dwi * e[0];
 #pragma unroll
         for (int b = 1; b < D; ++b) xg[b] += wi * e[b];
+      }
       }
 #pragma unroll
       for (int b = 0; b < D; ++b) {
@@ -1522,11 +1727,9 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     for (int i = 0; i < D; ++i)
 #pragma unroll
       for (int j = 0; j < D; ++j) E[i][j] = staged(stage, b + R::F + i * D + j) - (i == j ? P.f_diag : 0.0f);
-    p2g_pass<D, MAT, DET>(P, P.basis2, active, scene, p, x, v, C, E, staged(stage, b + R::Q),
-                          staged(stage, b + R::Q + 1), MAT == kMixed ? A.matid[p] : MAT, A.group, A.wact,
-                          scene_grid(A.PMm, scene, P), A.box_m + scene * 8, rec, sh.scatter[1],
-                          seen_m, err, A.Rm,
-                          nullptr, N);
+    p2g_pass<D, MAT, DET>(P, P.basis2, active, scene, p, staged_group(P, stage, Stage<D>::kAdj - 1), x, v, C, E,
+                          staged(stage, b + R::Q), staged(stage, b + R::Q + 1), MAT == kMixed ? A.matid[p] : MAT, A.wact,
+                          scene_grid(A.PMm, scene, P), A.box_m + scene * 8, rec, sh.scatter[1], seen_m, err, A.Rm, nullptr, N);
   }
   if (err) atomicOr(A.err, err);
 }
