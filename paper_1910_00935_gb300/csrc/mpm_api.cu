@@ -548,6 +548,7 @@ struct Launcher {
   // sequence: the next pass may then start while it drains (see pass_wait).  Anything else -- the
   // sequence's start, a clear, an event to wait for, a controller kernel -- is waited for in full.
   bool after_pass[2] = {false, false};
+  bool after_adjoint[2] = {false, false};  // and it was an adjoint pass: it writes no state
   int sid() const { return h->pm.sid; }
 
   // issue on the main (0) or the side (1) stream from now on
@@ -613,7 +614,10 @@ struct Launcher {
     ++count;
     const Dims& m = h->m;
     A.early = after_pass[sid()] && !h->profile;
+    if constexpr (std::is_same<Args, AdjArgs>::value)  // in 2D up to two waves of tiles (see adjoint_tile)
+      A.early_states = (!A.early || after_adjoint[sid()]) && (m.D == 3 || m.n_tiles <= 2 * 152 * (640 / MPM_TILE));
     after_pass[sid()] = true;
+    after_adjoint[sid()] = std::is_same<Args, AdjArgs>::value;
     return timed(category, [&] {
       if constexpr (std::is_same<Args, StepArgs>::value)
         return m.D == 2 ? launch_step<2>(h->desc.material, pmode, P, A, m.n_tiles, s)
@@ -794,6 +798,7 @@ struct Launcher {
     count += st ? 2 : 1;
     const bool early = after_pass[sid()] && !h->profile;
     after_pass[sid()] = true;
+    after_adjoint[sid()] = false;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_forward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off), st,
                                  h->at<int>(L.group), h->at<float>(L.ctrl_part), h->at<float>(L.wact),
@@ -815,6 +820,7 @@ struct Launcher {
     count += apply ? 2 : 1;
     const bool early = after_pass[sid()] && !h->profile;
     after_pass[sid()] = !apply;
+    after_adjoint[sid()] = false;
     return timed(MPM_KERNEL_CONTROLLER, [&] {
       return launch_ctrl_backward(c, m.S, m.n_tiles, m.N, h->at<int4>(L.tiles), h->at<int>(L.scene_tile_off),
                                   h->at<int>(L.group), h->at<float>(L.wbar_tile), h->at<float>(L.wact),

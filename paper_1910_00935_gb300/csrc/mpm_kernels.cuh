@@ -113,6 +113,7 @@ struct AdjArgs {
   unsigned* err;
   const float* sense_add;  // kAdjG2P: sensor adjoints [scene][slot][2D] added to xbar, vbar (or null)
   int early;  // launched as a programmatic dependent (host only)
+  int early_states;  // no state is written by a pass that may still run when this one starts
 };
 
 // Grid reads in the particle passes.  A grid written by an earlier launch is read through
@@ -1131,60 +1132,63 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   const int nranks = A.scene_tiles[scene];
   float* stage = reinterpret_cast<float*>(rec) + Rec<D>::kFloats;
   if (P.n_groups > 0) stage_row(stage, Stage<D>::kAdj - 1, reinterpret_cast<const float*>(A.group) + p);
-  if (NC) pass_wait();
-  const int seen_ub = MODE != kAdjP2G && A.box_ub ? box_seen(A.box_ub + scene * 8) : 0;
-  const int seen_m = MODE != kAdjP2G && A.stm ? box_seen(A.box_m + scene * 8) : 0;
-  stage_clears(A.clears, scene, sh.clear_box);
   stage_commit();
-  if (tile.w == 0) {
-    reset_box(A.box_ub_reset, scene);
-    reset_box(A.box_m_reset, scene);
-  }
-  // stage what the G2P-adjoint (state s: x, F) and the recomputed P2G (state s-1, mu, la)
-  // read, so that those loads are in flight during the P2G-adjoint
-  if (MODE != kAdjP2G) {
-#pragma unroll
-    for (int a = 0; a < D; ++a) stage_row(stage, a, A.st0 + (int64_t)(R::X + a) * N + p);
-#pragma unroll
-    for (int i = 0; i < D * D; ++i) stage_row(stage, D + i, A.st0 + (int64_t)(R::F + i) * N + p);
-  }
-  stage_commit();
+
+  constexpr bool kStress = MODE != kAdjG2P;
+  constexpr bool kLate = D == 3;
   constexpr bool kCarried = D == 3 && MODE != kAdjG2P;
   constexpr int kSums = D + 2 * D * D;
   static_assert(D == 2 || kSums + 4 <= Stage<D>::kAdj - 1 - Stage<D>::kAdjB, "the carried rows fit");
-  if (MODE != kAdjP2G && A.stm) {  // the recomputed P2G runs whenever state s-1 is given
-#pragma unroll
-    for (int r = 0; r < R::Q; ++r) stage_row(stage, Stage<D>::kAdjB + r, A.stm + (int64_t)r * N + p);
-    stage_row(stage, Stage<D>::kAdjB + R::Q, A.mu + p);
-    stage_row(stage, Stage<D>::kAdjB + R::Q + 1, A.la + p);
-  }
-  // without it, its rows hold what the P2G-adjoint needs after its gather: the carried adjoint, C
-  // of state s+1, the material sums -- at four CTAs an SM each exposed round trip is ~3% of a
-  // tile's 33,000 cycles (with the group ahead of the chain and nothing waiting for the dL/dw
-  // slot, 16 x 65,536 fixed-corotated: fused pass 263 -> 250 us, last P2G-adjoint 215 -> 199)
   const bool carried = kCarried && !A.stm;
-  if (carried) {
-    constexpr int b = Stage<D>::kAdjB;
-#pragma unroll
-    for (int a = 0; a < D; ++a) stage_row(stage, b + a, A.adj + (int64_t)(R::X + a) * N + p);
-#pragma unroll
-    for (int i = 0; i < D * D; ++i) {
-      stage_row(stage, b + D + i, A.adj + (int64_t)(R::F + i) * N + p);
-      stage_row(stage, b + D + D * D + i, A.st1 + (int64_t)(R::C + i) * N + p);
+  int seen_ub = 0, seen_m = 0;
+  auto stage_rest = [&]() {
+    seen_ub = MODE != kAdjP2G && A.box_ub ? box_seen(A.box_ub + scene * 8) : 0;
+    seen_m = MODE != kAdjP2G && A.stm ? box_seen(A.box_m + scene * 8) : 0;
+    stage_clears(A.clears, scene, sh.clear_box);
+    stage_commit();
+    if (tile.w == 0) {
+      reset_box(A.box_ub_reset, scene);
+      reset_box(A.box_m_reset, scene);
     }
-    stage_pair(stage, b + kSums, A.mubar + p);
-    stage_pair(stage, b + kSums + 2, A.labar + p);
-  }
-  stage_commit();
-
+    // stage what the G2P-adjoint (state s: x, F) and the recomputed P2G (state s-1, mu, la)
+    // read, so that those loads are in flight during the P2G-adjoint
+    if (MODE != kAdjP2G) {
+#pragma unroll
+      for (int a = 0; a < D; ++a) stage_row(stage, a, A.st0 + (int64_t)(R::X + a) * N + p);
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) stage_row(stage, D + i, A.st0 + (int64_t)(R::F + i) * N + p);
+    }
+    stage_commit();
+    if (MODE != kAdjP2G && A.stm) {  // the recomputed P2G runs whenever state s-1 is given
+#pragma unroll
+      for (int r = 0; r < R::Q; ++r) stage_row(stage, Stage<D>::kAdjB + r, A.stm + (int64_t)r * N + p);
+      stage_row(stage, Stage<D>::kAdjB + R::Q, A.mu + p);
+      stage_row(stage, Stage<D>::kAdjB + R::Q + 1, A.la + p);
+    }
+    // without it, its rows hold what the P2G-adjoint needs after its gather: the carried adjoint, C
+    // of state s+1, the material sums -- at four CTAs an SM each exposed round trip is ~3% of a
+    // tile's 33,000 cycles (with the group ahead of the chain and nothing waiting for the dL/dw
+    // slot, 16 x 65,536 fixed-corotated: fused pass 263 -> 250 us, last P2G-adjoint 215 -> 199)
+    if (carried) {
+      constexpr int b = Stage<D>::kAdjB;
+#pragma unroll
+      for (int a = 0; a < D; ++a) stage_row(stage, b + a, A.adj + (int64_t)(R::X + a) * N + p);
+#pragma unroll
+      for (int i = 0; i < D * D; ++i) {
+        stage_row(stage, b + D + i, A.adj + (int64_t)(R::F + i) * N + p);
+        stage_row(stage, b + D + D * D + i, A.st1 + (int64_t)(R::C + i) * N + p);
+      }
+      stage_pair(stage, b + kSums, A.mubar + p);
+      stage_pair(stage, b + kSums + 2, A.labar + p);
+    }
+    stage_commit();
+  };
   // adjoint of state s+1: xb, vb, Cb, Fb (Fb = dL/dE = dL/dF); C1 = C of state s+1.  In 3D,
   // after a P2G-adjoint the carried xb, Fb and the rows of state s+1 needed again (C, E,
   // mu, la, the polar factor) are read after its gather -- fresh loads, as the gather's
   // barriers order them -- so that none of them holds a register across the gather (in 2D
   // they fit: loaded once, before it)
-  constexpr bool kLate = D == 3;
-  float xb[D], vb[D], Cb[D][D], Fb[D][D];
-  float C1[D][D];
+  float xb[D], vb[D], Cb[D][D], Fb[D][D], C1[D][D];
   auto load_carried = [&]() {
     if (carried) {
       stage_wait<0>();
@@ -1205,11 +1209,70 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
 #pragma unroll
       for (int j = 0; j < D; ++j) {
         Fb[i][j] = A.adj[(R::F + i * D + j) * N + p];
-        C1[i][j] = A.st1[(R::C + i * D + j) * N + p];
+        if (kLate || !kStress) C1[i][j] = A.st1[(R::C + i * D + j) * N + p];
       }
   };
 
-  if (MODE == kAdjG2P || !kLate) load_carried();
+  // State s+1 and its stress: a quarter of a tile's time that needs nothing of the pass before when
+  // that is an adjoint pass (states are written by step passes: early_states).  It then goes ahead
+  // of the wait, its rows read through the L2 (nothing that an SM kept from another pass).  Forward
+  // and reverse: 49,152 liquid particles over 256 steps 6.38 -> 5.97 ms, 3,477 in 2D over 384 steps
+  // 3.93 -> 3.72, the 262,144-particle neo-Hookean cube 28.68 -> 28.17.  2D passes of many waves
+  // lose 1% (the launch decides); 3D fixed-corotated ones lose 0.5% (the rows are read again
+  // after the gather, then from the L1) and keep the wait first.
+  constexpr bool kMayLead = NC && kStress && (D == 2 || MAT == kNeoHookean || MAT == kLiquid);
+  const bool early = kMayLead && A.early_states;
+  if (!early) {
+    if (NC) pass_wait();
+    stage_rest();
+    if (MODE == kAdjG2P || !kLate) load_carried();
+  }
+  float x[D], v[D], E[D][D], Am[D][D], mv[D];
+  Axes<D> s;
+  StressCache<D> sc;
+  bool ok = false;
+  int axis = 0, grp = -1, mat_p = MAT;
+  float act = 0.0f;
+  if constexpr (kStress) {
+    auto row = [&](int r) {
+      const float* at = A.st1 + (int64_t)r * N + p;
+      return kMayLead ? __ldcg(at) : *at;
+    };
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      x[a] = row(R::X + a);
+      v[a] = row(R::V + a);
+    }
+#pragma unroll
+    for (int i = 0; i < D * D; ++i) {
+      E[i / D][i % D] = row(R::F + i) - (i / D == i % D ? P.f_diag : 0.0f);
+      C1[i / D][i % D] = row(R::C + i);
+    }
+    const float mu = A.mu[p], la = A.la[p];
+    ok = make_axes<D>(x, P, s) && active;
+    if (active && !ok) err |= kErrOOB;
+    if (early) stage_wait<0>();  // this thread's group
+    else stage_wait<3>();
+    grp = staged_group(P, stage, Stage<D>::kAdj - 1);
+    act = particle_act(P, P.basis, grp, A.wact, scene, D, axis);
+    float tau[D][D];
+    if (MAT == kMixed) mat_p = A.matid[p];
+    if (!kirchhoff<D, MAT>(E, mu, la, act, axis, tau, sc, A.R1, N, p, mat_p) && ok) {
+      err |= kErrNonFinite;
+      ok = false;
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      mv[i] = P.p_mass * v[i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) Am[i][j] = P.kappa * tau[i][j] + P.p_mass * C1[i][j];
+    }
+    if (early) {
+      pass_wait();
+      stage_rest();
+      if (!kLate) load_carried();
+    }
+  }
   if (MODE == kAdjG2P) {
 #pragma unroll
     for (int a = 0; a < D; ++a) vb[a] = A.adj[(R::V + a) * N + p];
@@ -1227,36 +1290,6 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
   } else {
     // ---- P2G adjoint of step s+1: gather (pbar, mbar) = grid_op.grad(ubar, (m, p)) ----
-    float x[D], v[D], E[D][D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      x[a] = A.st1[(R::X + a) * N + p];
-      v[a] = A.st1[(R::V + a) * N + p];
-    }
-    load_E<D>(A.st1, N, p, P.f_diag, E);
-    Axes<D> s;
-    bool ok = make_axes<D>(x, P, s) && active;
-    if (active && !ok) err |= kErrOOB;
-    int axis;
-    stage_wait<2>();  // this thread's group and its share of the clear boxes, before the barrier below
-    const int grp = staged_group(P, stage, Stage<D>::kAdj - 1);
-    const float act = particle_act(P, P.basis, grp, A.wact, scene, D, axis);
-    const float mu = A.mu[p], la = A.la[p];
-    float tau[D][D];
-    StressCache<D> sc;
-    const int mat_p = MAT == kMixed ? A.matid[p] : MAT;
-    if (!kirchhoff<D, MAT>(E, mu, la, act, axis, tau, sc, A.R1, N, p, mat_p) && ok) {
-      err |= kErrNonFinite;
-      ok = false;
-    }
-    float Am[D][D], mv[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      mv[i] = P.p_mass * v[i];
-#pragma unroll
-      for (int j = 0; j < D; ++j)
-        Am[i][j] = P.kappa * tau[i][j] + P.p_mass * (kLate ? A.st1[(R::C + i * D + j) * N + p] : C1[i][j]);
-    }
     float Ab[D][D], xg[D], sw[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -1274,8 +1307,10 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     gbx.use_tile = false;
     if (P.gather_capacity > 0) {
       gbx = box_extent<D>(ok, s.base, P.gather_capacity, sh.gather[0]);
+      stage_wait<2>();  // this thread's share of the clear boxes, before the box's barrier
       box_load<D, 2>(gbx, reinterpret_cast<float4*>(sm), P, raw, pbar);
     } else {
+      stage_wait<2>();
       __syncthreads();
     }
     run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);

@@ -1,7 +1,7 @@
 // setup.cu -- one-time set-up, permutation, loss and output kernels.
 //
-// Particles are reordered once per mpm_set_initial by (scene, Morton code of the
-// initial stencil base) so that every P2G tile covers a compact block of cells; an elastic
+// Particles are reordered once per mpm_set_initial by (scene, runs of 8 cells along the last
+// axis, the runs in Morton order) so that every P2G tile covers a compact block of cells; an elastic
 // body keeps its neighbours, so the order stays coherent for the whole run and the
 // tape never has to record a permutation.  Every input is gathered into that order
 // and every output scattered back to the caller's.
