@@ -603,10 +603,12 @@ def fp64_roofline(mpm, workload, category, n_launch, cat_ms, particles_per_launc
 
 
 def scatter_roofline(mpm, prof, N, dim):
-    """Grid reductions per second of the scattering passes against this GPU's float4
-    reduction rate measured live (mpm_measure_peak): one float4 reduction per particle and
-    stencil node (3^dim), the work that bounds these L2-resident passes rather than bytes.
-    The recomputed P2G of a resident segment's adjoint passes is not counted."""
+    """Contributions to the grid per second of the scattering passes (one per particle and
+    stencil node, 3^dim) against this GPU's float4 reduction rate measured live
+    (mpm_measure_peak). The passes add up the contributions of neighbouring particles before
+    they reduce (6-8 reductions a particle are left in 3D, ~4 in 2D), so this is the rate that
+    one reduction per contribution would need, and it may exceed the peak. The recomputed P2G
+    of a resident segment's adjoint passes is not counted."""
     red = mpm.mpm_measure_peak(mpm.MPM_PEAK_RED_F32X4)
     spread = mpm.mpm_measure_peak(mpm.MPM_PEAK_RED_F32X4_SPREAD)
     out = {"bound": "l2_reductions", "unit": "float4 reductions/s", "peak": red,
