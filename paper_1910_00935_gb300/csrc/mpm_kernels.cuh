@@ -483,8 +483,8 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
 //   vec   W * (a + B dpos)
 // A particle's 3^D nodes are 3^(D-1) columns along the grid's last axis.  Each warp scatters
 // its own 32 particles: lane (slot, column) walks its slot's third (3D) or eighth (2D) of them
-// in order, sums their contributions to its column's three nodes in registers, and while the
-// stencil base moves along the last axis by a node or two only reduces the nodes that fall out
+// in order, sums their contributions to its column's three nodes in registers, and where the
+// stencil base moves by one node along the last axis reduces only the node that falls out
 // of the window into the grid; any other move reduces all three.  The particle order makes
 // runs of such moves (sort_keys_kernel), but nothing depends on it.
 //
@@ -503,7 +503,7 @@ __device__ __forceinline__ void with_nodes(const BoxInfo<D>& b, const float4* sm
 
 // Write this thread's scatter record: the B-spline weights per axis, the affine value at the
 // stencil's centre node a + B dpos(1, 1, 1), its increment per node B dx, and the packed base
-// (-1: no scatter; its weights and values are then zero).  Every thread writes its record.
+// (-1: no scatter, whatever its weights and values).  Every thread writes its record.
 template <int D>
 __device__ __forceinline__ void put_record(float4* rec, bool valid, const Axes<D>& s, const float a[D],
                                            const float B[D][D], float dx) {
@@ -610,7 +610,7 @@ __device__ __forceinline__ void scatter_runs(const float4* rec, float4* g, int n
   a0.zero();
   a1.zero();
   a2.zero();
-  int cur = -1, node = 0;
+  int cur = -2, node = 0;  // (no base, nor the -1 of a refused particle: even a walk's first record is compared)
 #pragma unroll 1
   for (; r < end; ++r) {
     const float* w0 = reinterpret_cast<const float*>(r);
