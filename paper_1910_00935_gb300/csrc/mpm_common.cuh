@@ -194,17 +194,9 @@ __host__ __device__ __forceinline__ float ll_to_float_rn(long long a) {
 
 // the fixed-point node as floats: channel 0 times u0, the others times u1 (powers of two,
 // so each product is exact and the node value is rounded once, in ll_to_float_rn)
-template <bool NC>
 __device__ __forceinline__ float4 fix_load(const float4* g, int64_t node, float u0, float u1) {
   const longlong2* q = reinterpret_cast<const longlong2*>(g + 2 * node);
-  longlong2 a, b;
-  if (NC) {
-    a = __ldg(q);
-    b = __ldg(q + 1);
-  } else {
-    a = q[0];
-    b = q[1];
-  }
+  const longlong2 a = q[0], b = q[1];
   return make_float4(ll_to_float_rn(a.x) * u0, ll_to_float_rn(a.y) * u1, ll_to_float_rn(b.x) * u1,
                      ll_to_float_rn(b.y) * u1);
 }

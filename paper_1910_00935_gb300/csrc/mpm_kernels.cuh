@@ -116,36 +116,30 @@ struct AdjArgs {
   int early_states;  // no state is written by a pass that may still run when this one starts
 };
 
-// Grid reads in the particle passes.  A grid written by an earlier launch is read through
-// the read-only data path (NC); inside a persistent launch the grid was written by an
-// earlier pass of the same launch, so it is read with coherent loads, which the barrier's
-// acquire makes current.
-template <bool NC>
-__device__ __forceinline__ float4 grid_load(const float4* p) {
-  if (NC) return __ldg(p);
-  return *p;
-}
-
-// node `node` of a scene's (m, p) grid as floats (DET: fixed-point grid)
-template <bool NC, bool DET>
+// Grid reads in the particle passes are ordinary (coherent) loads: a pass may be resident while
+// the pass before it still scatters into the grid that it will gather (see pass_wait), or run in
+// the same persistent launch, so the read-only path (__ldg), which is defined for memory that nothing
+// writes while a kernel runs and whose loads may be moved above the wait, is not for them.
+// Node `node` of a scene's (m, p) grid as floats (DET: fixed-point grid).
+template <bool DET>
 __device__ __forceinline__ float4 pm_load(const float4* g, int64_t node, const SimParams& P) {
-  if (DET) return fix_load<NC>(g, node, P.unfix_m, P.unfix_p);
-  return grid_load<NC>(g + node);
+  if (DET) return fix_load(g, node, P.unfix_m, P.unfix_p);
+  return g[node];
 }
 // fixed-point scale pair of this backward's velocity-adjoint grids (deterministic mode)
 __device__ __forceinline__ void ub_scales(const unsigned* m0, float& fix, float& unfix) {
   fix_scales_from(__uint_as_float(*(const volatile unsigned*)m0), fix, unfix);
 }
 // node of a scene's velocity-adjoint grid
-template <bool NC, bool DET>
+template <bool DET>
 __device__ __forceinline__ float4 ub_load(const float4* g, int64_t node, const SimParams& P,
                                           const unsigned* m0) {
   if (DET) {
     float fix, unfix;
     ub_scales(m0, fix, unfix);
-    return fix_load<NC>(g, node, unfix, unfix);
+    return fix_load(g, node, unfix, unfix);
   }
-  return grid_load<NC>(g + node);
+  return g[node];
 }
 // Programmatic launch: a pass may start while the pass before it on its stream drains.  wait: every
 // access to what another pass writes comes after it (it returns once that pass has completed and
@@ -905,14 +899,15 @@ __device__ __forceinline__ void p2g_pass(const SimParams& P, const float* basis,
 // forward particle pass: [G2P of step t-1] then [P2G of step t]
 // ---------------------------------------------------------------------------
 // One tile of a forward pass; every thread of the CTA calls it.  sm: dynamic shared memory
-// (step_smem_bytes).  A CTA that runs several tiles must synchronise between them.
+// (step_smem_bytes).  OWN: the pass is a launch of its own (it then waits for the one before it), not
+// one of a persistent launch.  A CTA that runs several tiles must synchronise between them.
 //
 // A tile is a chain of dependent round trips to the L2 -- its entry, its particles' rows, its
 // box of grid nodes -- and a 2,048-tile cube runs in two waves of 7 tiles per SM, so what is
 // not part of the chain stays off it: the clear jobs' boxes, mu and la come by asynchronous
 // copies, the bounds of a box need one barrier and no reset, all nodes of a box are read
 // before the first is used, and a warp scatters without waiting for the others.
-template <int D, int MAT, int MODE, bool NC, bool DET>
+template <int D, int MAT, int MODE, bool OWN, bool DET>
 __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A, int tile_index,
                                           float* sm, TileShared& sh) {
   using R = Rows<D>;
@@ -933,7 +928,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
   }
   if (P.n_groups > 0) stage_row(stage, 2, reinterpret_cast<const float*>(A.group) + p);
   const int nranks = A.scene_tiles[scene];
-  if (NC) pass_wait();
+  if (OWN) pass_wait();
   const int seen = MODE != kG2POnlyFull ? box_seen(A.box_w + scene * 8) : 0;
   // the particle's rows first: in flight while the clears below read their boxes
   float x[D], v[D], C[D][D], E[D][D];
@@ -970,7 +965,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     }
     const float4* PMg = scene_grid(A.PMr, scene, P);
     stage_wait<0>();  // (this thread's share of the clear boxes, before the barrier below)
-    auto raw = [&](int f) { return pm_load<NC, DET>(PMg, f, P); };
+    auto raw = [&](int f) { return pm_load<DET>(PMg, f, P); };
     auto velocity = [&](float4 pm, bool wall) { return node_velocity<D>(pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
@@ -984,7 +979,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
     } else {
       __syncthreads();
     }
-    if (NC) pass_ready();
+    if (OWN) pass_ready();
     run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
     if (ok) {
       // centred on the stencil's centre node: equal because sum W dpos = 0, and
@@ -1081,7 +1076,7 @@ __device__ __forceinline__ void step_tile(const SimParams& P, const StepArgs& A,
                   A.sense + (int64_t)tile_index * (P.n_groups + 1) * (2 * D + 1));
   if (MODE != kG2POnlyFull) {
     stage_wait<0>();
-    if (NC && MODE == kP2GOnly) pass_ready();
+    if (OWN && MODE == kP2GOnly) pass_ready();
     p2g_pass<D, MAT, DET>(P, P.basis, active, scene, p, staged_group(P, stage, 2), x, v, C, E, staged(stage, 0),
                           staged(stage, 1), MAT == kMixed ? A.matid[p] : MAT, A.wact, scene_grid(A.PMw, scene, P), A.box_w + scene * 8, rec, sh.scatter[0], seen, err, nullptr, A.Rw, N);
     if (MODE == kP2GOnly) run_clears<D>(A.clears, sh.clear_box, scene, tile.w, nranks, P.nnodes, n);
@@ -1115,7 +1110,7 @@ __global__ void __launch_bounds__(kTile, step_ctas_per_sm<D, MAT>())
 // [recomputed P2G of step s-1, the grid the next adjoint pass needs (Appendix D.1)]
 // ---------------------------------------------------------------------------
 // One tile of an adjoint pass (same calling rules as step_tile; s_wbar: kWbarSlots floats).
-template <int D, int MAT, int MODE, bool NC, bool DET>
+template <int D, int MAT, int MODE, bool OWN, bool DET>
 __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& A, int tile_index,
                                              float* sm, TileShared& sh, float* s_wbar) {
   using R = Rows<D>;
@@ -1220,10 +1215,10 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
   // 3.93 -> 3.72, the 262,144-particle neo-Hookean cube 28.68 -> 28.17.  2D passes of many waves
   // lose 1% (the launch decides); 3D fixed-corotated ones lose 0.5% (the rows are read again
   // after the gather, then from the L1) and keep the wait first.
-  constexpr bool kMayLead = NC && kStress && (D == 2 || MAT == kNeoHookean || MAT == kLiquid);
+  constexpr bool kMayLead = OWN && kStress && (D == 2 || MAT == kNeoHookean || MAT == kLiquid);
   const bool early = kMayLead && A.early_states;
   if (!early) {
-    if (NC) pass_wait();
+    if (OWN) pass_wait();
     stage_rest();
     if (MODE == kAdjG2P || !kLate) load_carried();
   }
@@ -1301,7 +1296,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
     const float4* UBg = scene_grid(A.UB1, scene, P);
     const float4* PMg = scene_grid(A.PM1, scene, P);
-    auto raw = [&](int f) { return NodePair{ub_load<NC, DET>(UBg, f, P, A.ub_m0), pm_load<NC, DET>(PMg, f, P)}; };
+    auto raw = [&](int f) { return NodePair{ub_load<DET>(UBg, f, P, A.ub_m0), pm_load<DET>(PMg, f, P)}; };
     auto pbar = [&](const NodePair& g, bool wall) { return node_adjoint<D>(g.ub, g.pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;
@@ -1543,7 +1538,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
     }
   }
 
-  if (NC) pass_ready();
+  if (OWN) pass_ready();
   // ---- G2P adjoint of step s: x' = x + dt v', E' = E + dt C' (I + E) ----
   {
     float x0[D], E0[D][D];
@@ -1601,7 +1596,7 @@ __device__ __forceinline__ void adjoint_tile(const SimParams& P, const AdjArgs& 
       return;
     }
     const float4* PMg = scene_grid(A.PM0, scene, P);
-    auto raw = [&](int f) { return pm_load<NC, DET>(PMg, f, P); };
+    auto raw = [&](int f) { return pm_load<DET>(PMg, f, P); };
     auto velocity = [&](float4 pm, bool wall) { return node_velocity<D>(pm, wall, P); };
     BoxInfo<D> gbx;
     gbx.use_tile = false;

@@ -40,3 +40,24 @@ def test_equals_passes_one_by_one(mpm, name):  # noqa: F811
     want = grads(PROFILE=1)
     for options in ({}, {"USE_GRAPHS": 0}, {"OVERLAP_RESIM": 0}, {"GRID_RECOMPUTE": 1}, {"GRID_RECOMPUTE": 1, "OVERLAP_RESIM": 0}):
         assert all(torch.equal(a, b) for a, b in zip(grads(**options), want)), options
+
+
+@pytest.mark.parametrize("name", list(SCENES))
+def test_equals_passes_one_by_one_without_gather_box(mpm, name):  # noqa: F811
+    """Without the shared gather box a pass's grid reads hang on nothing but its particles' positions,
+    which an early pass has before the grid is written."""
+    scene, T = SCENES[name](), 7
+    scene["desc"]["deterministic_p2g"], scene["desc"]["ckpt_every"] = 1, 4
+    seeds = {k: torch.as_tensor(v).cuda() for k, v in _random_seeds(scene, np.random.default_rng(2)).items()}
+
+    def run(profile):
+        sim = mpm.from_scene(scene, max_steps=T)
+        sim.set_option(mpm.MPM_OPT_PROFILE, profile)
+        sim.set_option(mpm.MPM_OPT_GATHER_CAPACITY, 0)
+        sim.forward(T)
+        out = [t.clone() for t in sim.state()] + [t.clone() for t in sim.backward(**seeds).values()]
+        sim.check()
+        sim.close()
+        return out
+
+    assert all(torch.equal(a, b) for a, b in zip(run(0), run(1)))
