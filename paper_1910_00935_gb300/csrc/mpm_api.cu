@@ -261,6 +261,9 @@ struct mpm_handle {
   // grids only): (m, p) buffers res_lo .. res_lo + res_n - 1, each written once, its box in parity 0
   int res_lo = 0, res_n = 0;
   bool grids_clean = false;  // every other grid buffer holds zeros (false: the next set-up clears all)
+  // a call was captured into a graph of the caller's: it may be replayed at any time from then on,
+  // which this object does not see, so no sequence leaves grids for another any more
+  bool captured = false;
   // options
   bool use_graphs = true;
   bool smem_tile = false;  // with tile_capacity only checked against the device (see mpm.h)
@@ -889,8 +892,9 @@ struct Launcher {
 int last_segment_start(const mpm_handle* h, int T) { return ((T - 1) / h->m.K) * h->m.K; }
 
 // whether a segment's grids stay live for its adjoint passes: those of a re-simulated segment, and
-// those of the last segment from the forward that ran it
+// (leaves_grids) those of the last segment from the forward that ran it
 bool keeps_grids(const mpm_handle* h) { return h->m.store_grids && !h->grid_recompute; }
+bool leaves_grids(const mpm_handle* h) { return keeps_grids(h) && !h->captured; }
 
 // the (m, p) pool a forward's grid of step t is allocated from: the last segment's, which stay
 // live, in order from the start of the pool of that segment's parity, the others in the other pool
@@ -936,7 +940,7 @@ int issue_coarse_resim(mpm_handle* h, Launcher& Lc, int Jc, int T) {
 int issue_forward(mpm_handle* h, Launcher& Lc, int T) {
   const int K = h->m.K;
   const int sL = last_segment_start(h, T);
-  const bool keep = keeps_grids(h);
+  const bool keep = leaves_grids(h);
   ring_reset(h->pm);
   ring_reset(h->ub);
   const float* src = h->state(h->L.ckpt, 0);
@@ -1120,7 +1124,7 @@ int issue_backward(mpm_handle* h, Launcher& Lc, int T, bool resident, bool grids
 int issue_forward_ctrl(mpm_handle* h, Launcher& Lc, int T) {
   const int K = h->m.K;
   const int sL = last_segment_start(h, T);
-  const bool keep = keeps_grids(h);
+  const bool keep = leaves_grids(h);
   ring_reset(h->pm);
   ring_reset(h->ub);
   const float* src = h->state(h->L.ckpt, 0);
@@ -1209,8 +1213,20 @@ int issue_backward_ctrl(mpm_handle* h, Launcher& Lc, int T, bool resident, bool 
   return MPM_OK;
 }
 
-// Zero the grids that a forward left for its backward, where something else comes next.
-int drop_residents(mpm_handle* h, cudaStream_t s) {
+// Whether the caller is capturing `s` (the handle notes it for good).
+bool note_capture(mpm_handle* h, cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();  // (the legacy stream while another is captured: the call's own launches report it)
+    return false;
+  }
+  if (st != cudaStreamCaptureStatusNone) h->captured = true;
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// Zero the grids that a forward left for its backward, where something else comes next.  In a
+// capture the clear is only recorded: the grids are then still there for the next call made directly.
+int drop_residents(mpm_handle* h, cudaStream_t s, bool capturing) {
   if (h->res_n == 0) return MPM_OK;
   const Dims& m = h->m;
   Clears C;
@@ -1223,7 +1239,7 @@ int drop_residents(mpm_handle* h, cudaStream_t s) {
                            : launch_clear_run<3>(C, g, stride, b, 2 * m.S * 8, h->res_n, (int)m.nnodes, m.n_grid, m.S, s);
   if (e == cudaSuccess) e = launch_reset_boxes(b, (int64_t)h->res_n * 2 * m.S, s);
   h->launches += 2;
-  h->res_n = 0;
+  if (!capturing || e != cudaSuccess) h->res_n = 0;
   if (e != cudaSuccess) {
     h->grids_clean = false;
     return cuda_fail(h, e, "clearing the last forward's grids");
@@ -1515,15 +1531,18 @@ int mpm_set_initial(mpm_handle* h, const float* x0, const float* v0, const float
   // Every launch sequence leaves the grid buffers at zero but for the last forward's, so only the
   // first set-up (or one after a failure) clears them all: on a 262,144-particle cube that was
   // 4.6 GB, 0.7 ms of every set-up.
-  if (h->grids_clean) {
-    int rc = drop_residents(h, s);
+  const bool capturing = note_capture(h, s);
+  if (h->grids_clean && !capturing) {
+    int rc = drop_residents(h, s, false);
     if (rc) return rc;
   } else {
     const size_t grid = (size_t)m.S * m.nnodes * sizeof(float4) * m.words;
     CK(cudaMemsetAsync(h->at<char>(L.grids), 0, grid * (m.pm_slots + kUBSlots), s));
     CK(launch_reset_boxes(h->at<int>(L.boxes), (int64_t)(m.pm_slots + kUBSlots) * 2 * m.S, s));
-    h->res_n = 0;
-    h->grids_clean = true;
+    if (!capturing) {  // (a captured set-up has cleared nothing yet)
+      h->res_n = 0;
+      h->grids_clean = true;
+    }
   }
   CK(cudaMemsetAsync(h->at<char>(L.box_stats), 0, 16, s));
   ring_reset(h->pm);
@@ -1557,13 +1576,13 @@ int mpm_forward(mpm_handle* h, int32_t T, void* stream) {
   if (T < 1 || T > h->max_steps) return fail(h, MPM_ERR_STATE, "T must be in [1, max_steps]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   h->last_stream = s;
-  int rc = drop_residents(h, s);
+  int rc = drop_residents(h, s, note_capture(h, s));
   if (rc) return rc;
-  rc = run_sequence(h, (int64_t)T * 2, s, [&](Launcher& Lc) {
+  rc = run_sequence(h, (int64_t)T * 2 + (leaves_grids(h) ? 0 : ((int64_t)1 << 43)), s, [&](Launcher& Lc) {
     return h->m.ctrl_H > 0 ? issue_forward_ctrl(h, Lc, T) : issue_forward(h, Lc, T);
   });
   if (rc) return rc;
-  if (keeps_grids(h)) {
+  if (leaves_grids(h)) {
     h->res_lo = forward_pool(h, T, T - 1) * h->m.pm_pool;
     h->res_n = T - last_segment_start(h, T);
   }
@@ -1647,9 +1666,10 @@ int mpm_backward(mpm_handle* h, const float* dL_dx, const float* dL_dv, const fl
   h->launches += 4;
   const int T = h->T_recorded;
   const bool resident = h->resident_T == T;
-  const bool grids = resident && h->res_n > 0 && keeps_grids(h);
+  const bool capturing = note_capture(h, s);
+  const bool grids = resident && h->res_n > 0 && leaves_grids(h);
   if (!grids) {
-    int rc = drop_residents(h, s);
+    int rc = drop_residents(h, s, capturing);
     if (rc) return rc;
   }
   // the re-simulation overlaps the adjoint passes when there is a segment to re-simulate,
@@ -1667,7 +1687,7 @@ int mpm_backward(mpm_handle* h, const float* dL_dx, const float* dL_dv, const fl
   // the same forward re-simulates the last segment as well
   if (last_segment_start(h, T) > 0) {
     h->resident_T = 0;
-    h->res_n = 0;  // (cleared as its passes went)
+    if (grids) h->res_n = 0;  // (cleared as its passes went)
   }
   float* outs[4] = {gx0, gv0, gC0, gF0};
   r0 = 0;
@@ -1703,6 +1723,7 @@ int mpm_initial_p2g_grid(mpm_handle* h, float* grid, void* stream) {
     return fail(h, MPM_ERR_STATE, "MPM_MIXED: mpm_set_particle_materials has not been called");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   h->last_stream = s;
+  note_capture(h, s);
   Launcher Lc{h, s};
   ring_reset(h->pm);
   ring_reset(h->ub);

@@ -101,3 +101,73 @@ def test_diagnostic_grid_between(mpm):
         assert float((a - b).norm()) <= 1e-4 * max(float(b.norm()), 1e-30)
     assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
     sim.close()
+
+
+@pytest.mark.parametrize("name", ["cube", "rects", "nn"])
+@pytest.mark.parametrize("k", [4, 40])
+@pytest.mark.parametrize("before", [False, True])  # a forward whose kept grids the capture meets
+def test_calls_captured_by_the_caller(mpm, name, k, before):
+    """A caller's own graph of a call, replayed any number of times and between calls made directly,
+    gives what the call gives."""
+    scene = _scene(name)
+    scene["desc"]["ckpt_every"] = k
+    seeds = {key: torch.as_tensor(v).cuda() for key, v in _random_seeds(scene, np.random.default_rng(3)).items()}
+    ref_sim = mpm.from_scene(scene, max_steps=T)
+    ref_sim.forward(T)
+    x, ref = [t.clone() for t in ref_sim.state()], _back(ref_sim, seeds)
+
+    sim = mpm.from_scene(scene, max_steps=T)
+    sim.set_option(mpm.MPM_OPT_USE_GRAPHS, 0)  # (a library graph cannot be launched into a capture)
+    out = [torch.empty_like(t) for t in x]
+    g = {key: torch.empty_like(v) for key, v in ref_sim.backward(**seeds).items()}
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        sim.forward(T)
+        _back(sim, seeds)
+        if before:
+            sim.forward(T)
+    stream.synchronize()
+
+    def capture(fn):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            fn()
+        return graph
+
+    def backward():
+        mpm.mpm_backward(sim.h, **seeds, **{key: (v if v.numel() else None) for key, v in g.items()})
+
+    forward = capture(lambda: (mpm.mpm_forward(sim.h, T), mpm.mpm_get_state(sim.h, *out)))
+    both = capture(lambda: (mpm.mpm_forward(sim.h, T), backward()))
+    setup = capture(lambda: mpm.mpm_set_initial(sim.h, *sim._inputs))
+    sim.T = T
+
+    def replay(graph):
+        for t in out + list(g.values()):
+            t.fill_(float("nan"))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+
+    for _ in range(3):
+        replay(forward)
+        _same(out, x)
+    for _ in range(2):
+        replay(both)
+        _same(list(g.values()), ref)
+    replay(setup)
+    replay(forward)
+    _same(out, x)
+    sim.reload()
+    sim.forward(T)                      # called directly, a replay between it and its backward
+    replay(forward)
+    _same(_back(sim, seeds), ref)
+    replay(forward)
+    sim.forward(T)
+    _same(_back(sim, seeds), ref)
+    replay(both)
+    _same(list(g.values()), ref)
+    _same(_back(sim, seeds), ref)
+    assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
+    ref_sim.close()
+    sim.close()
