@@ -1805,7 +1805,11 @@ int mpm_set_option(mpm_handle* h, int32_t key, int64_t value) {
       if (value < 0 || value > 65535) return fail(h, MPM_ERR_ARG, "grid blocks must be in [0, 65535]");
       h->grid_blocks = (int)value;
       break;
-    case MPM_OPT_POLAR_CACHE: h->use_polar_cache = value != 0; break;
+    case MPM_OPT_POLAR_CACHE:
+      // a forward without the cache left no factors of its last segment: re-simulate that one too
+      if (h->m.polar_cache && value != 0 && !h->use_polar_cache) h->resident_T = 0;
+      h->use_polar_cache = value != 0;
+      break;
     case MPM_OPT_GRID_RECOMPUTE: h->grid_recompute = value != 0; break;
     case MPM_OPT_PERSISTENT: h->persistent = value != 0; break;
     case MPM_OPT_OVERLAP_RESIM: h->overlap = value != 0; break;

@@ -171,3 +171,25 @@ def test_calls_captured_by_the_caller(mpm, name, k, before):
     assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
     ref_sim.close()
     sim.close()
+
+
+@pytest.mark.parametrize("k", [4, 40])
+@pytest.mark.parametrize("first,then", [(0, 1), (1, 0)])
+def test_polar_cache_switched_between(mpm, k, first, then):
+    """The factors that a forward leaves for its backward are used only where it wrote them."""
+    scene = scenes.make("robots3d", n_scenes=2, dims=(12, 8, 8))
+    scene["desc"]["deterministic_p2g"], scene["desc"]["ckpt_every"] = 1, k
+    seeds = {key: torch.as_tensor(v).cuda() for key, v in _random_seeds(scene, np.random.default_rng(3)).items()}
+    ref_sim = mpm.from_scene(scene, max_steps=T)
+    ref_sim.forward(T)
+    ref = _back(ref_sim, seeds)
+    sim = mpm.from_scene(scene, max_steps=T)
+    sim.set_option(mpm.MPM_OPT_POLAR_CACHE, first)
+    sim.forward(T)
+    sim.set_option(mpm.MPM_OPT_POLAR_CACHE, then)
+    for _ in range(2):
+        for a, b in zip(_back(sim, seeds), ref):  # (a factor formed in another pass may round differently)
+            assert float((a - b).norm()) <= 1e-4 * float(b.norm())
+    assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
+    ref_sim.close()
+    sim.close()
