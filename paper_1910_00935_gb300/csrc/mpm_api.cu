@@ -261,6 +261,9 @@ struct mpm_handle {
   // grids only): (m, p) buffers res_lo .. res_lo + res_n - 1, each written once, its box in parity 0
   int res_lo = 0, res_n = 0;
   bool grids_clean = false;  // every other grid buffer holds zeros (false: the next set-up clears all)
+  // persistent launches were issued since the last status: one may have given up, its passes' clears
+  // undone, so a set-up does not rely on clean grids
+  bool unseen_waits = false;
   // a call was captured into a graph of the caller's: it may be replayed at any time from then on,
   // which this object does not see, so no sequence leaves grids for another any more
   bool captured = false;
@@ -1342,6 +1345,7 @@ int run_sequence_impl(mpm_handle* h, int64_t key, cudaStream_t stream, Fn&& issu
 // (which clears every buffer) before the next forward.
 template <typename Fn>
 int run_sequence(mpm_handle* h, int64_t key, cudaStream_t stream, Fn&& issue) {
+  if (h->persistent && h->m.ctrl_H == 0) h->unseen_waits = true;
   int rc = run_sequence_impl(h, key, stream, issue);
   if (rc != MPM_OK) {
     h->initialized = false;
@@ -1532,7 +1536,7 @@ int mpm_set_initial(mpm_handle* h, const float* x0, const float* v0, const float
   // first set-up (or one after a failure) clears them all: on a 262,144-particle cube that was
   // 4.6 GB, 0.7 ms of every set-up.
   const bool capturing = note_capture(h, s);
-  if (h->grids_clean && !capturing) {
+  if (h->grids_clean && !h->unseen_waits && !capturing) {
     int rc = drop_residents(h, s, false);
     if (rc) return rc;
   } else {
@@ -1542,6 +1546,7 @@ int mpm_set_initial(mpm_handle* h, const float* x0, const float* v0, const float
     if (!capturing) {  // (a captured set-up has cleared nothing yet)
       h->res_n = 0;
       h->grids_clean = true;
+      h->unseen_waits = false;
     }
   }
   CK(cudaMemsetAsync(h->at<char>(L.box_stats), 0, 16, s));
@@ -1748,6 +1753,7 @@ int mpm_sync_status(mpm_handle* h) {
   unsigned err = 0;
   e = cudaMemcpy(&err, h->at<unsigned>(h->L.err), 4, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(h, e, "read error word");
+  h->unseen_waits = false;
   if (err) {
     cudaMemset(h->at<unsigned>(h->L.err), 0, 4);
     // a timeout first: the passes after the barrier that gave up never ran, so whatever else

@@ -193,3 +193,28 @@ def test_polar_cache_switched_between(mpm, k, first, then):
     assert mpm.mpm_sync_status(sim.h) == mpm.MPM_OK
     ref_sim.close()
     sim.close()
+
+
+def test_set_up_after_a_wait_that_gave_up_unseen(mpm):
+    """A persistent forward whose barrier gives up leaves grids half written; a set-up clears them even if
+    nobody asked for the status in between."""
+    scene = scenes.make("square2d", n_side=32)
+    scene["desc"]["deterministic_p2g"], scene["desc"]["ckpt_every"] = 1, 4  # (no grid of the early steps is kept)
+    ref = mpm.from_scene(scene, max_steps=T)
+    ref.forward(T)
+    x = [t.clone() for t in ref.state()]
+    sim = mpm.from_scene(scene, max_steps=T)
+    sim.forward(T)  # (the grids are known to be clean from here on)
+    first = list(sim._inputs)
+    sim.set_initial(first[0] + 0.02, first[1] + 1.0, *first[2:6])
+    sim.set_option(mpm.MPM_OPT_PERSISTENT, 1)
+    sim.set_option(mpm.MPM_OPT_BARRIER_TIMEOUT_US, 20000)
+    sim.set_option(mpm.MPM_OPT_BARRIER_TEST_EXTRA, 1)  # an arrival that never comes
+    sim.forward(T)
+    sim.set_option(mpm.MPM_OPT_PERSISTENT, 0)
+    sim.set_initial(*first[:6])
+    sim.forward(T)
+    _same(sim.state(), x)
+    assert mpm.mpm_sync_status(sim.h) == mpm.MPM_ERR_TIMEOUT  # (the wait that gave up is still reported)
+    ref.close()
+    sim.close()
