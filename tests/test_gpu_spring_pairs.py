@@ -74,3 +74,26 @@ def test_zero_length_spring_is_finite(ms):
     sim.close()
     assert float(x.abs().max()) == 0.0 and float(v.abs().max()) == 0.0
     assert all(bool(torch.isfinite(t).all()) for t in (gx, gv, gl))
+
+
+@pytest.mark.parametrize("dim,n", [(2, 2), (3, 3), (3, 6)])
+def test_nan_reaches_every_axis_of_a_spring(ms, dim, n):
+    """A coordinate that is not a number makes its spring's length, and so all axes of the force on both
+    ends (and of their adjoints), not a number; other systems stay clear of it."""
+    S, springs = 5, [(j, j + 1) for j in range(n - 1)]
+    x0 = torch.arange(n * dim, dtype=torch.float32, device="cuda")[:, None].repeat(1, S) * 0.1
+    v0 = torch.zeros_like(x0)
+    rest = torch.full((n - 1, S), 0.2, device="cuda")
+    x0[0, 2] = float("nan")
+    sim = ms.MassSprings(dim, n, springs, S, 50.0, 1.0, 1e-3, steps=2)
+    sim.forward(x0, v0, rest, 2)
+    x, v = sim.state()
+    gx, gv, gl = sim.backward(torch.ones_like(x0), torch.ones_like(x0))
+    sim.sync()
+    sim.close()
+    hit = torch.zeros(n * dim, S, dtype=torch.bool, device="cuda")
+    hit[:2 * dim, 2] = True  # the two ends of the first spring
+    assert torch.equal(torch.isnan(x), hit) and torch.equal(torch.isnan(v), hit)
+    assert torch.equal(torch.isnan(gx), hit)
+    assert not bool(torch.isnan(gv).any())  # one step back: v0 reaches the state through x alone
+    assert torch.equal(torch.isnan(gl), torch.nn.functional.one_hot(torch.tensor(2), S).bool().cuda() & (torch.arange(n - 1).cuda() == 0)[:, None])
