@@ -97,3 +97,17 @@ def test_nan_reaches_every_axis_of_a_spring(ms, dim, n):
     assert torch.equal(torch.isnan(gx), hit)
     assert not bool(torch.isnan(gv).any())  # one step back: v0 reaches the state through x alone
     assert torch.equal(torch.isnan(gl), torch.nn.functional.one_hot(torch.tensor(2), S).bool().cuda() & (torch.arange(n - 1).cuda() == 0)[:, None])
+
+
+@pytest.mark.parametrize("n", [2, 6])
+def test_force_beyond_the_range_is_infinite(ms, n):
+    """k times the strain above FP32's range: the force is infinite along the spring, as the quotient is."""
+    x0 = torch.zeros(2 * n, 3, device="cuda")
+    x0[2] = 1e10  # mass 1, along x
+    sim = ms.MassSprings(2, n, [(0, 1)], 3, 1e30, 1.0, 1e-3, steps=2)
+    sim.forward(x0, torch.zeros_like(x0), torch.zeros(1, 3, device="cuda"), 2)
+    x, v = sim.state()
+    sim.sync()
+    sim.close()
+    assert bool((v[0] == float("inf")).all()) and bool((v[2] == -float("inf")).all())
+    assert bool((x[0] == float("inf")).all()) and bool((x[2] == -float("inf")).all())
