@@ -3,6 +3,8 @@ the kernels), in either order of a spring's ends, for each kernel variant (at mo
 springs unrolled or looped, up to 8 masses) and batch size (blocks of 128 and of 512 threads),
 against the FP64 oracle on sampled systems; a spring of zero length stays finite."""
 import itertools
+import os
+import subprocess
 
 import numpy as np
 import pytest
@@ -111,3 +113,17 @@ def test_force_beyond_the_range_is_infinite(ms, n):
     sim.close()
     assert bool((v[0] == float("inf")).all()) and bool((v[2] == -float("inf")).all())
     assert bool((x[0] == float("inf")).all()) and bool((x[2] == -float("inf")).all())
+
+
+def test_roots_and_quotients_round_as_derived(tmp_path):
+    """spring_math.cuh over every length it can meet: half an ulp plus the second-order term of one
+    correction (below 2^-19 ulp; asserted at 2^-18); the reciprocal root within CUDA's 2 ulp."""
+    from paper_1910_00935_gb300 import build
+    exe = str(tmp_path / "spring_math_check")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "host", "spring_math_check.cu")
+    subprocess.run([build.nvcc(), *build.ARCH, "-std=c++17", "-O2", "-o", exe, src], check=True, capture_output=True, timeout=300)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=300).stdout
+    err = {line.split()[0]: float(line.split()[1]) for line in out.strip().splitlines()}
+    for name in ("sqrt", "rcp", "div"):
+        assert err[name] <= 0.5 + 2.0 ** -18, out
+    assert err["rsqrt"] <= 2.0, out
