@@ -11,8 +11,8 @@
 //
 // Weights arrive in FP32; a tile's sensor sums are FP32, the sums over tiles and the dot products
 // compensated FP32 pairs (value and correction, ~48 bits: FP64 runs at 1/64 of the FP32 rate on
-// this part, and a few thousand FP64 operations a step were most of these kernels' time), the
-// inputs and what is kept for the reverse FP64, the activations tanh in FP32.  Every sum runs in a
+// this part, and a few thousand FP64 operations a step were most of these kernels' time; a sum that
+// leaves FP32's range is formed again in FP64), the inputs and what is kept for the reverse FP64, the activations tanh in FP32.  Every sum runs in a
 // fixed order (a warp's lanes by butterfly, a tile's warps and a scene's tiles in order), so the
 // controller adds nothing order-dependent to a deterministic run.
 //
@@ -22,6 +22,8 @@
 // adjoint adds the sensors' adjoints as it reads the state's (AdjArgs::sense_add).  Measured on
 // 4 x 27,648 particles, 32 hidden units (us a launch under ncu): sensing 8.3 -> in the G2P pass, MLP
 // 19.3 -> 10.6, reverse 25.5 -> 14.5, adding the sensors' adjoints 7.3 -> in the adjoint pass.
+#include <cfloat>
+
 #include "mpm_internal.h"
 #include "mpm_kernels.cuh"
 
@@ -56,6 +58,8 @@ __device__ __forceinline__ Pair pair_mul(float w, Pair u) {  // w * (h + l)
   two_prod(w, u.h, p, e);
   return pair_norm(p, fmaf(w, u.l, e));
 }
+// whether a sum stayed within FP32's range (once beyond it, a pair never comes back)
+__device__ __forceinline__ bool in_range(Pair a) { return fabsf(a.h) <= FLT_MAX; }
 // sum over the lanes of aligned groups of LANES, the same order on every run (all lanes call it)
 template <int LANES>
 __device__ __forceinline__ Pair lanes_sum(Pair v) {
@@ -63,6 +67,22 @@ __device__ __forceinline__ Pair lanes_sum(Pair v) {
   for (int o = LANES / 2; o > 0; o >>= 1)
     v = pair_add(v, {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
   return v;
+}
+
+// sum over i < n of w[i * stride] * u[i] in FP64 by a whole warp: the way out of a pair that left its
+// range (out of line: what never happens in earnest holds no registers)
+__device__ __noinline__ double dot_fp64(const float* w, int stride, const double* u, int n) {
+  double z = 0.0;
+  for (int i = threadIdx.x & 31; i < n; i += 32) z += (double)w[i * stride] * u[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  return z;
+}
+// sum over t in [t0, t1) of a[t * nv] in FP64 by one thread
+__device__ __noinline__ double rows_fp64(const float* a, int t0, int t1, int nv) {
+  double z = 0.0;
+  for (int t = t0; t < t1; ++t) z += (double)a[(int64_t)t * nv];
+  return z;
 }
 
 // out[j] = sum over t in [t0, t1) of a[t * nv + j] for j < nv, by the whole CTA: thread (r, j)
@@ -87,10 +107,7 @@ __device__ void block_tile_sums(float* a, int t0, int t1, int nv, Pair* scratch,
         q[u] = in ? *e : 0.0f;
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (CLEAR && t + u * R < t1) a[(int64_t)(t + u * R) * nv + j] = 0.0f;
-        acc = pair_add(acc, {q[u], 0.0f});
-      }
+      for (int u = 0; u < U; ++u) acc = pair_add(acc, {q[u], 0.0f});
     }
   }
   scratch[threadIdx.x] = acc;
@@ -102,9 +119,11 @@ __device__ void block_tile_sums(float* a, int t0, int t1, int nv, Pair* scratch,
     if (v < nv)
       for (int k = q4 * per; k < R && k < (q4 + 1) * per; ++k) p = pair_add(p, scratch[k * nv + v]);
     p = lanes_sum<4>(p);
-    if (v < nv && q4 == 0) out[v] = pair_value(p);
+    if (v < nv && q4 == 0) out[v] = in_range(p) ? pair_value(p) : rows_fp64(a + v, t0, t1, nv);
   }
   __syncthreads();
+  if (CLEAR)
+    for (int64_t e = (int64_t)t0 * nv + threadIdx.x; e < (int64_t)t1 * nv; e += blockDim.x) a[e] = 0.0f;
 }
 
 // Per-tile sensor sums of the initial state (every later state's come from its G2P pass)
@@ -193,9 +212,11 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_forward_kernel(CtrlStep cs,
       if (i < n_in) z = pair_add(z, pair_mul(j == warp ? w1[q] : W1[j * n_in + i], u[i]));
     }
     z = pair_add(lanes_sum<32>(z), {j == warp ? bias1 : b1[j], 0.0f});
+    float zj = z.h + z.l;
+    if (!in_range(z)) zj = (float)(dot_fp64(W1 + j * n_in, 1, u_out + (int64_t)s * n_in, n_in) + (double)b1[j]);
     if (lane == 0) {
       // the activation in FP32: FP64 transcendentals run on the FP64 pipe
-      const float hj = tanhf(z.h + z.l);
+      const float hj = tanhf(zj);
       hs[j] = hj;
       h_out[(int64_t)s * H + j] = (double)hj;
     }
@@ -207,8 +228,10 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_forward_kernel(CtrlStep cs,
     for (int q = 0; q < 2; ++q)
       if (lane + 32 * q < H) z = pair_add(z, pair_mul(w2[q], {hs[lane + 32 * q], 0.0f}));
     z = pair_add(lanes_sum<32>(z), {bias2, 0.0f});
+    float zg = z.h + z.l;
+    if (!in_range(z)) zg = (float)(dot_fp64(W2 + warp * H, 1, h_out + (int64_t)s * H, H) + (double)bias2);
     if (lane == 0) {
-      const double y = (double)tanhf(z.h + z.l);
+      const double y = (double)tanhf(zg);
       y_out[(int64_t)s * G + warp] = y;
       act_out[(int64_t)s * G + warp] = (float)((double)cs.scale * y);
     }
@@ -293,7 +316,8 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_backward_kernel(CtrlStep cs
     for (int k = 0; k < 2; ++k)
       if (lane + 32 * k < H) acc = pair_add(acc, pair_mul(w1[q][k], z1p[lane + 32 * k]));
     acc = lanes_sum<32>(acc);
-    if (lane == 0) ub[i] = pair_value(acc);
+    const double ubi = in_range(acc) ? pair_value(acc) : dot_fp64(W1 + i, n_in, z1b, H);
+    if (lane == 0) ub[i] = ubi;
   }
   // the weights' adjoints: nothing below reads them
   for (int e = tid; e < G * H; e += kCtrlThreads) W2b[e] += z2b[e / H] * hsd[e % H];

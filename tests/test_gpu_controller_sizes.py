@@ -62,3 +62,25 @@ def test_scene_alone_and_in_a_batch(mpm):
         alone = _run_gpu(mpm, subset_scenes(scene, [i]), T, loss=False)["state"]
         for w, a in zip(whole, alone):
             assert np.array_equal(w[:, scene_slice(scene, i)], a)
+
+
+def test_hidden_units_beyond_the_range(mpm):
+    """A hidden unit's argument above FP32's range saturates it, as a smaller one of its sign does."""
+    T = 8
+
+    def run(w):
+        scene = _scene(3, 2, 2, 8, (6, 5))
+        scene["desc"].update(deterministic_p2g=1, act_phase=0.3)
+        n_in = 2 + 2 * 3 * 2
+        th = scene["arrays"]["w"].copy()
+        for j in range(8):  # the time inputs' weights, one sign a unit
+            th[:, j * n_in:j * n_in + 2] = w if j % 2 else -w
+        scene["arrays"]["w"] = th
+        seeds = _random_seeds(scene, np.random.default_rng(7))
+        return _run_gpu(mpm, scene, T, seeds=seeds, loss=False)
+
+    got, want = run(3e38), run(1e30)
+    for a, b in zip(got["state"], want["state"]):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
+    for key in got["grad"]:
+        assert np.array_equal(got["grad"][key], want["grad"][key]), key
