@@ -253,6 +253,7 @@ struct mpm_handle {
   char* ws = nullptr;
   size_t ws_bytes = 0;
   int smem_optin = 0;  // the device's per-CTA shared-memory limit (bytes)
+  int n_sm = 152;      // and its SMs
   bool initialized = false;
   bool materials_set = false;  // MPM_MIXED: per-particle materials given since the last set-up
   int32_t T_recorded = 0;
@@ -621,7 +622,7 @@ struct Launcher {
     const Dims& m = h->m;
     A.early = after_pass[sid()] && !h->profile;
     if constexpr (std::is_same<Args, AdjArgs>::value)  // in 2D up to two waves of tiles (see adjoint_tile)
-      A.early_states = (!A.early || after_adjoint[sid()]) && (m.D == 3 || m.n_tiles <= 2 * 152 * (640 / MPM_TILE));
+      A.early_states = (!A.early || after_adjoint[sid()]) && (m.D == 3 || m.n_tiles <= 2 * h->n_sm * MPM_ADJ_CTAS_PER_SM_2D);
     after_pass[sid()] = true;
     after_adjoint[sid()] = std::is_same<Args, AdjArgs>::value;
     return timed(category, [&] {
@@ -1466,6 +1467,11 @@ int mpm_create(const mpm_scene_desc* desc, void* workspace, size_t workspace_byt
     cudaGetLastError();
     h->smem_optin = 0;  // unknown: capacities are then checked by the launches alone
   }
+  int n_sm = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, attr.device) == cudaSuccess && n_sm > 0)
+    h->n_sm = n_sm;
+  else
+    cudaGetLastError();
   h->pm.n = m.pm_slots;
   h->ub.first = m.pm_slots;
   {
