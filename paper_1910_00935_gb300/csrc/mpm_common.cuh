@@ -46,6 +46,11 @@ namespace mpm {
 // adjoint passes: 2D 5 CTAs per SM (96 registers); 3D 4 (128 registers, no spills), which became
 // the faster one once the passes were shorter (fused adjoint, 262,144-particle neo-Hookean cube
 // 83 -> 81 us, 16 x 65,536 fixed-corotated 337 -> 318; in 2D 5 stays 10% faster)
+// (MPM_ADJ_CTAS_PER_SM sets both)
+#ifdef MPM_ADJ_CTAS_PER_SM
+#define MPM_ADJ_CTAS_PER_SM_2D MPM_ADJ_CTAS_PER_SM
+#define MPM_ADJ_CTAS_PER_SM_3D MPM_ADJ_CTAS_PER_SM
+#endif
 #ifndef MPM_ADJ_CTAS_PER_SM_2D
 #define MPM_ADJ_CTAS_PER_SM_2D (640 / MPM_TILE)
 #endif

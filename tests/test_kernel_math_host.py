@@ -57,3 +57,17 @@ def test_fixed_point_conversions_match_the_c_library(tmp_path):
     n, bad_round, bad_float = map(int, subprocess.run([exe], check=True, capture_output=True,
                                                       text=True, timeout=300).stdout.split())
     assert n > 0 and bad_round == 0 and bad_float == 0, (n, bad_round, bad_float)
+
+
+def test_build_macro_of_the_adjoint_occupancy(tmp_path):
+    """-DMPM_ADJ_CTAS_PER_SM sets the resident blocks of the adjoint passes in both dimensions; the macro
+    of one dimension alone leaves the other at its default."""
+    cc = _nvcc()
+    if cc is None:
+        pytest.skip("nvcc not found")
+    src = tmp_path / "macro.cu"
+    src.write_text(f'#include "{os.path.dirname(HERE)}/paper_1910_00935_gb300/csrc/mpm_common.cuh"\n'
+                   "static_assert(MPM_ADJ_CTAS_PER_SM_2D == WANT_2D && MPM_ADJ_CTAS_PER_SM_3D == WANT_3D);\n")
+    for flags, want in (([], (5, 4)), (["-DMPM_ADJ_CTAS_PER_SM=3"], (3, 3)), (["-DMPM_ADJ_CTAS_PER_SM_3D=2"], (5, 2))):
+        subprocess.run([cc, "-std=c++17", "--expt-relaxed-constexpr", *flags, f"-DWANT_2D={want[0]}", f"-DWANT_3D={want[1]}",
+                        "-c", "-o", str(tmp_path / "macro.o"), str(src)], check=True, capture_output=True, timeout=300)
