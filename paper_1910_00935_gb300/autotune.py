@@ -1,17 +1,19 @@
 """Autotuner for the launch knobs of libmpm (measurement-based, cached).
 
 The knobs are the library's runtime options: the capacity of the shared gather box
-(MPM_OPT_GATHER_CAPACITY), the particle order (MPM_OPT_SORT_ORDER), the options of earlier scatter
-forms, which the library accepts without effect (MPM_OPT_SMEM_TILE, MPM_OPT_BUCKET_SCATTER,
-MPM_OPT_PAIR_SCATTER, MPM_OPT_TILE_CAPACITY), the CTA count of the end-of-sequence grid clear (MPM_OPT_GRID_BLOCKS), the launch form
+(MPM_OPT_GATHER_CAPACITY), the particle order (MPM_OPT_SORT_ORDER), the CTA count of the
+end-of-sequence grid clear (MPM_OPT_GRID_BLOCKS), the launch form
 (MPM_OPT_PERSISTENT: one launch per pass, or persistent launches over the pass plan), and two
 memory-vs-recompute choices of the backward: a re-simulated segment's grids kept or recomputed
 per step (MPM_OPT_GRID_RECOMPUTE) and the re-simulation overlapped with the adjoint passes on a
 second stream or run before them (MPM_OPT_OVERLAP_RESIM).  `tune` times a short forward+backward
 of the caller's own simulator for each candidate, one knob at a time (coordinate descent
 from the defaults), keeps the fastest, and caches the result in a JSON file keyed by the
-workload's shape class and the device name.  Results never change numerics beyond FP32
-atomic-order rounding (the GPU tests check every knob setting against the oracle).
+workload's shape class and the device name.  The options of earlier scatter forms
+(MPM_OPT_SMEM_TILE, MPM_OPT_BUCKET_SCATTER, MPM_OPT_PAIR_SCATTER, MPM_OPT_TILE_CAPACITY), which the
+library accepts without effect, keep their places in a configuration but are not timed.
+Results never change numerics beyond FP32 atomic-order rounding (the GPU tests check every knob
+setting against the oracle).
 
 `tune_build` does the same for the build-time shapes: particles (= threads) per CTA,
 `MPM_TILE`, with the CTAs per SM of each pass that follow from it.  Each candidate is a
@@ -37,6 +39,7 @@ SPACE = {
     "grid_recompute": [0, 1],
     "overlap_resim": [1, 0],
 }
+NO_EFFECT = ("smem_tile", "bucket_scatter", "pair_scatter", "tile_capacity")
 DEFAULTS = {"gather_capacity": 512, "smem_tile": 0, "bucket_scatter": 0, "pair_scatter": 0, "sort_order": 0,
             "tile_capacity": 1024,
             "grid_blocks": 0,
@@ -150,7 +153,7 @@ def tune(sim, T: int = 32, repeats: int = 2, cache_path: str | None = None, forc
             failed.append([dict(config), str(e)])
             return float("inf")
 
-    config, t, log = coordinate_descent(measure)
+    config, t, log = coordinate_descent(measure, {k: v for k, v in SPACE.items() if k not in NO_EFFECT})
     sim.autotune_failed = failed
     apply(sim, config)
     if "sort_order" not in config and getattr(sim, "_inputs", None) is not None:

@@ -103,3 +103,17 @@ def test_tune_build_selection_validation_and_cache(tmp_path, monkeypatch):
     n = len(built)
     assert autotune.tune_build(scene, T=4, space=space, cache_path=cache, device_name="fake-gpu")["tag"] == "tile64"
     assert len(built) == n
+
+
+@pytest.mark.gpu
+def test_tune_times_no_option_without_effect(tmp_path):
+    from paper_1910_00935_gb300 import build, mpm, scenes
+    build.build()
+    sim = mpm.from_scene(scenes.make("square2d", n_side=16), max_steps=4)
+    path = str(tmp_path / "c.json")
+    cfg = autotune.tune(sim, T=4, repeats=1, cache_path=path)
+    sim.close()
+    (entry,) = autotune.load_cache(path).values()
+    for knob in ("smem_tile", "bucket_scatter", "pair_scatter", "tile_capacity"):
+        assert cfg[knob] == autotune.DEFAULTS[knob]
+        assert all(c[knob] == autotune.DEFAULTS[knob] for c, _ in entry["evaluated"])
