@@ -611,11 +611,15 @@ def scatter_roofline(mpm, prof, N, dim):
     of a resident segment's adjoint passes is not counted."""
     red = mpm.mpm_measure_peak(mpm.MPM_PEAK_RED_F32X4)
     spread = mpm.mpm_measure_peak(mpm.MPM_PEAK_RED_F32X4_SPREAD)
-    out = {"bound": "l2_reductions", "unit": "float4 reductions/s", "peak": red,
+    out = {"bound": None, "unit": "contributions/s", "peak": red,
+           "note": "achieved counts contributions (particle x stencil node); they are merged before the "
+                   "reduction, so frac is not a share of the reduction rate and may exceed 1",
            "peak_spread": spread,
            "peak_source": "measured live: mpm_measure_peak (float4 reductions, 32 lanes on 32 "
                           "consecutive nodes; peak_spread: on 32 cache lines)",
-           "reductions_per_particle": 3 ** dim, "kernels": {}}
+           "contributions_per_particle": 3 ** dim,
+           "reductions_per_particle": 3 ** dim,  # (if none were merged)
+           "kernels": {}}
     for cat in ("g2p_p2g", "g2p_p2g_full", "adj_fused"):
         if cat in prof and prof[cat][0]:
             n, ms = prof[cat]

@@ -33,8 +33,14 @@
  *     are sticky in the handle and reported by mpm_sync_status().
  *   - Ownership: the library allocates no device memory.  The caller provides one
  *     device workspace (size from mpm_workspace_bytes) at create time and owns it;
- *     it must outlive the handle.  Inputs are copied into the workspace; outputs
- *     go to caller-allocated buffers.  The handle itself is a small host object.
+ *     it must outlive the handle, which keeps tables, states and cleared grids in it
+ *     between calls: nothing else writes to it meanwhile.  Inputs are copied into the
+ *     workspace; outputs go to caller-allocated buffers.  The handle itself is a small
+ *     host object.
+ *   - With MPM_OPT_USE_GRAPHS 0 the calls that only launch (mpm_set_initial, mpm_forward,
+ *     mpm_get_state, mpm_loss, mpm_backward) may be captured into a graph of the
+ *     caller's; from the first captured one on, a forward leaves no grids for its
+ *     backward (see MPM_INFO_KEEPS_SEGMENT_GRIDS for those within a backward).
  */
 #ifndef MPM_H_
 #define MPM_H_

@@ -551,9 +551,10 @@ struct Launcher {
   cudaStream_t main_s = nullptr;  // (the caller's stream may be the legacy default, null)
   bool main_known = false;
   int pm_lo = 0, pm_hi = -1;
-  // whether the last operation issued on a stream (main, side) was a particle pass of this
-  // sequence: the next pass may then start while it drains (see pass_wait).  Anything else -- the
-  // sequence's start, a clear, an event to wait for, a controller kernel -- is waited for in full.
+  // whether the last operation issued on a stream (main, side) was a particle pass or a controller
+  // kernel of this sequence: the next pass may then start while it drains (see pass_wait).  Anything
+  // else -- the sequence's start, a clear, an event to wait for, the kernel that adds the first state's
+  // sensor adjoints -- is waited for in full.
   bool after_pass[2] = {false, false};
   bool after_adjoint[2] = {false, false};  // and it was an adjoint pass: it writes no state
   int sid() const { return h->pm.sid; }
