@@ -390,10 +390,12 @@ def springs_workload(seed=0, S=1 << 20, T=256):
 
 
 def springs_digest():
-    """Digest of the mass-spring kernels' source (csrc/mass_spring.cu)."""
+    """Digest of the mass-spring kernels' sources (csrc/mass_spring.cu, csrc/spring_math.cuh)."""
     import hashlib
-    path = os.path.join(ROOT, "paper_1910_00935_gb300", "csrc", "mass_spring.cu")
-    return hashlib.sha256(open(path, "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in ("mass_spring.cu", "spring_math.cuh"):
+        h.update(open(os.path.join(ROOT, "paper_1910_00935_gb300", "csrc", name), "rb").read())
+    return h.hexdigest()[:16]
 
 
 def springs_traffic(kernel, T):
