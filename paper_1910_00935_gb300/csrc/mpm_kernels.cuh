@@ -116,16 +116,23 @@ struct AdjArgs {
   int early_states;  // no state is written by a pass that may still run when this one starts
 };
 
-// Grid reads in the particle passes are ordinary (coherent) loads: a pass may be resident while
-// the pass before it still scatters into the grid that it will gather (see pass_wait), or run in
-// the same persistent launch, so the read-only path (__ldg), which is defined for memory that nothing
-// writes while a kernel runs and whose loads may be moved above the wait, is not for them.  (Nor is it
-// faster: 262,144-particle cube, 256 steps and reverse 28.3 ms through it, 27.9 without.)
+// Grid reads in the particle passes are coherent loads: a pass may be resident while the pass
+// before it still scatters into the grid that it will gather (see pass_wait), or run in the same
+// persistent launch, so the read-only path (__ldg), which is defined for memory that nothing writes while
+// a kernel runs and whose loads may be moved above the wait, is not for them.  As one ordered
+// 16-byte load they take the same time as through that path (1,024 steps and reverse of a
+// 262,144-particle cube 95.4 ms both, its first 256 steps 8.30, 16 x 65,536 fixed-corotated 57.3); left to
+// the compiler they gain 1.5% on the two shorter runs and lose 2.4% on the long forward (27.1 -> 27.8 ms).
+__device__ __forceinline__ float4 grid_load(const float4* p) {
+  float4 r;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p) : "memory");
+  return r;
+}
 // Node `node` of a scene's (m, p) grid as floats (DET: fixed-point grid).
 template <bool DET>
 __device__ __forceinline__ float4 pm_load(const float4* g, int64_t node, const SimParams& P) {
   if (DET) return fix_load(g, node, P.unfix_m, P.unfix_p);
-  return g[node];
+  return grid_load(g + node);
 }
 // fixed-point scale pair of this backward's velocity-adjoint grids (deterministic mode)
 __device__ __forceinline__ void ub_scales(const unsigned* m0, float& fix, float& unfix) {
@@ -140,7 +147,7 @@ __device__ __forceinline__ float4 ub_load(const float4* g, int64_t node, const S
     ub_scales(m0, fix, unfix);
     return fix_load(g, node, unfix, unfix);
   }
-  return g[node];
+  return grid_load(g + node);
 }
 // Programmatic launch: a pass may start while the pass before it on its stream drains.  wait: every
 // access to what another pass writes comes after it (it returns once that pass has completed and
