@@ -89,10 +89,8 @@ __device__ __noinline__ double rows_fp64(const float* a, int t0, int t1, int nv)
 // out[j] = sum over t in [t0, t1) of a[t * nv + j] for j < nv, by the whole CTA: thread (r, j)
 // sums rows t0 + r, t0 + r + R, ... (R = blockDim / nv, all reads issued before the first sum),
 // then four lanes a value sum its R partials in order and combine.  The order depends only on
-// (t0, t1), so the sums are reproducible.  CLEAR: zero every element read (the per-tile
-// actuation adjoints are consumed).  scratch: kCtrlThreads pairs; out: shared, nv doubles.
+// (t0, t1), so the sums are reproducible.  scratch: kCtrlThreads pairs; out: shared, nv doubles.
 // 4 nv <= blockDim.  Ends with a barrier.
-template <bool CLEAR>
 __device__ void block_tile_sums(float* a, int t0, int t1, int nv, Pair* scratch, double* out) {
   const int R = blockDim.x / nv;
   const int r = threadIdx.x / nv, j = threadIdx.x - r * nv;
@@ -123,8 +121,6 @@ __device__ void block_tile_sums(float* a, int t0, int t1, int nv, Pair* scratch,
     if (v < nv && q4 == 0) out[v] = in_range(p) ? pair_value(p) : rows_fp64(a + v, t0, t1, nv);
   }
   __syncthreads();
-  if (CLEAR)
-    for (int64_t e = (int64_t)t0 * nv + threadIdx.x; e < (int64_t)t1 * nv; e += blockDim.x) a[e] = 0.0f;
 }
 
 // Per-tile sensor sums of the initial state (every later state's come from its G2P pass)
@@ -177,7 +173,7 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_forward_kernel(CtrlStep cs,
   const int t0 = tile_off[s], t1 = tile_off[s + 1];
   pass_wait();
   pass_ready();
-  block_tile_sums<false>(part, t0, t1, ns * nv, scratch, sums);
+  block_tile_sums(part, t0, t1, ns * nv, scratch, sums);
   if ((int)threadIdx.x < ns) {
     const int g = threadIdx.x;
     double n = sums[g * nv + 2 * dim];
@@ -287,7 +283,7 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_backward_kernel(CtrlStep cs
     }
   pass_wait();
   pass_ready();
-  block_tile_sums<true>(abar_tile, t0, t1, G, scratch, abar);
+  block_tile_sums(abar_tile, t0, t1, G, scratch, abar);
   if (tid < G) {
     const double zb = abar[tid] * (double)cs.scale * (1.0 - y * y);
     z2b[tid] = zb;
@@ -340,6 +336,8 @@ __global__ void __launch_bounds__(kCtrlThreads) ctrl_backward_kernel(CtrlStep cs
     if (sl > 0) v += ub[K + (sl - 1) * 2 * dim + c] * inv_n[sl];
     add[((int64_t)s * ns + sl) * 2 * dim + c] = (float)v;
   }
+  // the tile slots, consumed, start the next step at zero
+  for (int64_t e = (int64_t)t0 * G + tid; e < (int64_t)t1 * G; e += kCtrlThreads) abar_tile[e] = 0.0f;
 }
 
 // xbar_p += add[scene][slot(p)][0..d), vbar_p += add[scene][slot(p)][d..2d): one CTA per
