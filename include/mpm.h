@@ -98,7 +98,9 @@ extern "C" {
                                      read the grid through L1 [512] */
 #define MPM_OPT_POLAR_CACHE 7     /* 3D fixed-corotated: the re-simulation stores each state's
                                      polar factor and F - R (FP32) for the two backward
-                                     passes that need them instead of recomputing them [1] */
+                                     passes that need them instead of recomputing them [1];
+                                     switched on between a forward and its backward, the last
+                                     segment is re-simulated as well */
 #define MPM_OPT_GRID_BLOCKS 6     /* CTAs per scene of the end-of-sequence grid clear; 0 = automatic [0] */
 #define MPM_OPT_PERSISTENT 8      /* 1: each run of passes of one kind and one pass mode (the
                                      fused steps of a forward; the re-simulation and the
